@@ -45,7 +45,7 @@ void launch_disp_group_norm(const double alpha[3], const double beta[3][3], cons
                             double dt, const double dx[3], int dims, const int N[3], int weight,
                             double wparam, double* scratch, double** out_dev, cudaStream_t st);
 size_t norm_scratch_doubles(const int N[3], long long npts);
-int diag_blocks(const Geom& g);
+size_t diag_scratch_bytes(const Geom& g);
 void launch_omega(const double alpha[3], const double beta[3][3], const double delta[3], double dt,
                   const double dx[3], int dims, const double* k_dev, int n, double* out_dev,
                   cudaStream_t st);
@@ -267,7 +267,7 @@ struct fdtd_handle {
     cudaEvent_t filled[2];   // ordering events between the handle's stream and the copy stream
     long long step;
     int use_fused;
-    double* dpart;      // diagnostics partials (3 per block)
+    double* dpart;      // diagnostics scratch (block ticket, phase tables, partials)
     std::vector<FusedMaps> hist_maps;   // TMA descriptors of each history snapshot (FP32 adjoint)
     FusedMaps lam_maps;                 // .e[c]: TMA descriptors of lambda_B component c (FP32)
     bool lam_staged = false;            // lam_maps valid: the staged FP32 adjoint E kernel runs
@@ -1049,7 +1049,13 @@ int fdtd_step_adjoint(fdtd_handle* h, int32_t n, const fdtd_probe* probe, double
 
 static int ensure_dpart(fdtd_handle* h) {
     if (h->dpart) return FDTD_OK;
-    CK(cudaMalloc(&h->dpart, (size_t)diag_blocks(h->g) * 3 * sizeof(double)));
+    CK(cudaMalloc(&h->dpart, diag_scratch_bytes(h->g)));
+    cudaError_t e = cudaMemsetAsync(h->dpart, 0, 16, h->stream);   // the block ticket
+    if (e != cudaSuccess) {
+        cudaFree(h->dpart);
+        h->dpart = nullptr;
+        CK(e);
+    }
     return FDTD_OK;
 }
 

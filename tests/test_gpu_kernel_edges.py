@@ -1,0 +1,80 @@
+"""Edge sizes of the kernels' tiles, items and dispatch rules against plain FP64 references."""
+import math
+
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+pytestmark = pytest.mark.gpu
+
+
+def _sim(shape, dtype="f32", dims=3, **kw):
+    from paper_1710_06829_gb300 import inputs
+    from paper_1710_06829_gb300 import sim as S
+    beta, delta = inputs.isotropic_theta(-0.05, -0.04, 0.02, 0.01)
+    return S.Simulation(shape, [1.0, 1.0, 1.0], 0.4, beta, delta, dims=dims, dtype=dtype, **kw)
+
+
+def _random_state(shape, dtype, seed=0):
+    """Six seeded fields rounded to the dtype, as FP64 arrays."""
+    from paper_1710_06829_gb300 import inputs
+    np_t = np.float32 if dtype == "f32" else np.float64
+    return [f.astype(np_t).astype(np.float64) for f in inputs.random_fields(shape, seed)]
+
+
+# one row, one column group, a ragged last item (17 rows), several planes, more items than a wave
+PROJECTION_SHAPES = [((4, 1, 1), 1), ((8, 17, 1), 2), ((12, 16, 5), 3), ((68, 33, 3), 3),
+                     ((256, 130, 40), 3)]
+
+
+@pytest.mark.parametrize("dtype", ["f32", "f64"])
+@pytest.mark.parametrize("shape,dims", PROJECTION_SHAPES)
+def test_projections_match_direct_sums(shape, dims, dtype):
+    """Plane-wave amplitude, energy moments and window energy against direct FP64 sums.  The sums
+    have n terms of relative error a few eps, so n eps sum|term| bounds the difference; 1e-13
+    sum|term| (about 500 eps) holds with room for the pairwise-like order used."""
+    from paper_1710_06829_gb300 import inputs
+    nx, ny, nz = shape
+    f = _random_state(shape, dtype)
+    sm = _sim(shape, dtype, dims)
+    sm.set_state([torch.from_numpy(a) for a in f])
+    for comp, k in ((0, (0.3, -0.7, 1.1)), (5, (2.9, 0.01, -3.0))):
+        x, y, z = inputs.positions(shape, comp, [1.0, 1.0, 1.0])
+        ref = np.sum(f[comp] * np.exp(-1j * (k[0] * x + k[1] * y + k[2] * z)))
+        for _ in range(2):   # the block ticket is back at zero after the first launch
+            got = sm.plane_wave(comp, k).cpu().numpy()
+            assert abs(got[0] + 1j * got[1] - ref) <= 1e-13 * np.sum(np.abs(f[comp]))
+    for axis in range(3):
+        n = shape[axis]
+        ref = np.zeros(3)
+        for c in range(6):
+            th = 2 * math.pi * inputs.positions(shape, c, [1.0, 1.0, 1.0])[axis] / n
+            e = 0.5 * f[c] ** 2
+            ref += [e.sum(), (e * np.cos(th)).sum(), (e * np.sin(th)).sum()]
+        got = sm.energy_moments(axis).cpu().numpy()
+        assert np.all(np.abs(got - ref) <= 1e-13 * ref[0])
+    ref = 0.5 * sum(np.sum(np.take(a, range(-3, nx - 4), axis=2, mode="wrap") ** 2) for a in f)
+    got = float(sm.energy(-3, nx - 1).cpu())
+    assert abs(got - ref) <= 1e-13 * ref
+    sm.close()
+
+
+def test_plane_wave_of_denormals_and_non_finite_values():
+    """The integer widening of the FP32 projection: denormal floats keep their values, an infinity or
+    a NaN reaches the sums as the plain conversion would bring it there."""
+    shape = (8, 20, 2)
+    f = torch.zeros((2, 20, 8), dtype=torch.float32)
+    f[1, 19, 5], f[0, 3, 2], f[1, 7, 0] = 3e-42, -1e-44, 2e-39
+    sm = _sim(shape)
+    for bad in (None, math.inf, math.nan):
+        if bad is not None:
+            f[0, 17, 6] = bad
+        sm.set_state([None, None, f, None, None, None])
+        re, im = sm.plane_wave(2, (0.0, 0.0, 0.0)).cpu().tolist()
+        ref = float(f.double().sum())
+        if bad is None:
+            assert abs(re - ref) <= 1e-15 * abs(ref) and im == 0.0
+        else:
+            assert math.isnan(re) if math.isnan(ref) else re == ref
+    sm.close()
