@@ -546,14 +546,21 @@ static int copy_in(fdtd_handle* h, void* const fields[6], int32_t mem, T* const 
         CK(cudaEventRecord(h->filled[1], h->xfer));
         CK(cudaStreamWaitEvent(h->stream, h->filled[1], 0));
     }
+    const T* src[6];
+    T* to[6];
+    int n = 0;
     for (int c = 0; c < 6; ++c) {
-        const T* src = (const T*)(fields ? fields[c] : nullptr);
-        if (src && mem == FDTD_MEM_HOST)
+        const T* f = (const T*)(fields ? fields[c] : nullptr);
+        if (f && mem == FDTD_MEM_HOST) {
             launch_fill_ghosts<T>(h->g, dst[c], h->stream);
-        else
-            launch_unpack<T>(h->g, src, dst[c], h->stream);   // NULL source: zeros
-        CK(cudaGetLastError());
+            CK(cudaGetLastError());
+            continue;
+        }
+        src[n] = f;   // NULL source: zeros
+        to[n++] = dst[c];
     }
+    launch_unpack<T>(h->g, src, to, n, h->stream);
+    CK(cudaGetLastError());
     if (mem == FDTD_MEM_HOST) CK(cudaStreamSynchronize(h->stream));
     return FDTD_OK;
 }
@@ -575,11 +582,16 @@ static int copy_out(fdtd_handle* h, void* const fields[6], int32_t mem, T* const
         CK(cudaStreamSynchronize(h->xfer));
         return FDTD_OK;
     }
+    const T* from[6];
+    T* out[6];
+    int n = 0;
     for (int c = 0; c < 6; ++c) {
         if (!fields[c]) continue;
-        launch_pack<T>(h->g, srcs[c], (T*)fields[c], h->stream);
-        CK(cudaGetLastError());
+        from[n] = srcs[c];
+        out[n++] = (T*)fields[c];
     }
+    launch_pack<T>(h->g, from, out, n, h->stream);
+    CK(cudaGetLastError());
     return FDTD_OK;
 }
 
@@ -719,9 +731,9 @@ static int ensure_jx(fdtd_handle* h, int n) {
 template <typename T>
 static int snapshot(fdtd_handle* h, int snap) {
     const size_t arr = (size_t)h->g.total * sizeof(T);
-    for (int c = 0; c < 3; ++c)
-        CK(cudaMemcpyAsync(h->hist_arr(snap, c), h->arr(h->cur, c), arr, cudaMemcpyDeviceToDevice,
-                           h->stream));
+    // the three components are adjacent in the state set and in the history
+    CK(cudaMemcpyAsync(h->hist_arr(snap, 0), h->arr(h->cur, 0), 3 * arr, cudaMemcpyDeviceToDevice,
+                       h->stream));
     return FDTD_OK;
 }
 
@@ -927,15 +939,13 @@ int fdtd_checkpoint(fdtd_handle* h, int32_t slot, int32_t op) {
     }
     if (op == 0) {
         if (!h->ckpt[slot]) CK(cudaMalloc(&h->ckpt[slot], 6 * arr));
-        for (int c = 0; c < 6; ++c)
-            CK(cudaMemcpyAsync(h->ckpt[slot] + c * arr, h->arr(h->cur, c), arr,
-                               cudaMemcpyDeviceToDevice, h->stream));
+        CK(cudaMemcpyAsync(h->ckpt[slot], h->arr(h->cur, 0), 6 * arr, cudaMemcpyDeviceToDevice,
+                           h->stream));   // a state set's six arrays are adjacent
         h->ckpt_step[slot] = h->step;
     } else {
         if (!h->ckpt[slot]) { set_error("checkpoint slot %d is empty", slot); return FDTD_ESTATE; }
-        for (int c = 0; c < 6; ++c)
-            CK(cudaMemcpyAsync(h->arr(h->cur, c), h->ckpt[slot] + c * arr, arr,
-                               cudaMemcpyDeviceToDevice, h->stream));
+        CK(cudaMemcpyAsync(h->arr(h->cur, 0), h->ckpt[slot], 6 * arr, cudaMemcpyDeviceToDevice,
+                           h->stream));
         h->step = h->ckpt_step[slot];
         h->hist_len = 0;
     }

@@ -150,10 +150,14 @@ void launch_probe_loss(const Geom& g, const T* E, int x_index, const T* target, 
 template <typename T>
 void launch_probe_adjoint(const Geom& g, T* lamE, const T* E, int x_index, const T* target,
                           cudaStream_t st);
+// n <= 6 arrays between the padded and the dense layout; unpacking writes the periodic images too,
+// and zeros where dense[i] is NULL
 template <typename T>
-void launch_pack(const Geom& g, const T* padded, T* dense, cudaStream_t st);
+void launch_pack(const Geom& g, const T* const padded[6], T* const dense[6], int n,
+                 cudaStream_t st);
 template <typename T>
-void launch_unpack(const Geom& g, const T* dense, T* padded, cudaStream_t st);
+void launch_unpack(const Geom& g, const T* const dense[6], T* const padded[6], int n,
+                   cudaStream_t st);
 // the periodic images (ghost cells) of a padded array from its owned cells
 template <typename T>
 void launch_fill_ghosts(const Geom& g, T* padded, cudaStream_t st);

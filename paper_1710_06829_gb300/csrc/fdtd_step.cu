@@ -339,41 +339,119 @@ template void launch_bunch_table<double>(int, int, double, double, double, doubl
 // layout conversion
 // ---------------------------------------------------------------------------
 
+// Up to six components in one launch (blockIdx.y), by chunks of V elements: V * sizeof(T) = 16
+// bytes when the dense pointers allow it (nx is a multiple of 4 and PX = 4, so a padded row splits
+// into whole chunks, and the image of a dense chunk is a whole chunk), single elements otherwise.
+// A block owns R whole rows, which are contiguous in the dense array; a thread moves COPY_ILP chunks
+// at a time, all loads before the stores, with one division by the row length a chunk.  The owner
+// of a chunk writes its images, so the dense array is read once.  256^3 FP32, six components, 805 MB
+// (119 us at the copy rate): unpacking took 556 us with one element and four 64-bit divisions a
+// thread, 147 us here; packing 416 us, now 159 us.
+constexpr int COPY_THREADS = 256, COPY_ILP = 4;
+
 template <typename T>
-__global__ void unpack_kernel(Geom g, const T* __restrict__ dense, T* __restrict__ padded) {
-    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= g.total) return;
-    const int ip = (int)(t % g.nxp);
-    const long long r = t / g.nxp;
-    const int jp = (int)(r % g.nyp);
-    const int k = (int)(r / g.nyp);
-    int i = (ip - PX) % g.nx;
-    if (i < 0) i += g.nx;
-    int j = (jp - PY) % g.ny;
-    if (j < 0) j += g.ny;
-    padded[t] = dense == nullptr ? T(0) : dense[((long long)k * g.ny + j) * g.nx + i];
+struct CopyList {
+    const T* src[6];   // NULL (unpacking only): zeros
+    T* dst[6];
+};
+
+template <typename T, int V>
+struct alignas(V * sizeof(T)) Chunk {
+    T v[V];
+};
+
+// dense -> padded, images included (TO_PADDED), or owned cells of padded -> dense
+template <typename T, int V, bool TO_PADDED>
+__global__ void __launch_bounds__(COPY_THREADS) layout_kernel(Geom g, CopyList<T> list, int R) {
+    using C = Chunk<T, V>;
+    const int nc = g.nx / V, gc = PX / V;   // chunks of a dense row, of a ghost edge
+    const long long rows = (long long)g.ny * g.nz;
+    const T* src = list.src[blockIdx.y];
+    T* dst = list.dst[blockIdx.y];
+    const long long r0 = (long long)blockIdx.x * R;
+    const unsigned n = (unsigned)(rows - r0 < R ? rows - r0 : R) * (unsigned)nc;
+    const int k0 = (int)(r0 / g.ny), j0 = (int)(r0 - (long long)k0 * g.ny);
+    const long long dense0 = r0 * g.nx;
+    // padded offset of the block's chunk t; its row j in the plane and column chunk c
+    auto place = [&](unsigned t, int& j, int& c) {
+        const int r = (int)(t / (unsigned)nc);
+        c = (int)(t - (unsigned)r * nc);
+        j = j0 + r;
+        const int dk = j / g.ny;
+        j -= dk * g.ny;
+        return pidx(g, c * V, j, k0 + dk);
+    };
+    for (unsigned t0 = threadIdx.x; t0 < n; t0 += COPY_THREADS * COPY_ILP) {
+        C v[COPY_ILP];
+#pragma unroll
+        for (int q = 0; q < COPY_ILP; ++q) {
+            const unsigned t = t0 + q * COPY_THREADS;
+            if (t >= n) continue;
+            if (!TO_PADDED) {
+                int j, c;
+                v[q] = *reinterpret_cast<const C*>(src + place(t, j, c));
+            } else if (src != nullptr) {
+                v[q] = *reinterpret_cast<const C*>(src + dense0 + (long long)t * V);
+            } else {
+#pragma unroll
+                for (int u = 0; u < V; ++u) v[q].v[u] = T(0);
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < COPY_ILP; ++q) {
+            const unsigned t = t0 + q * COPY_THREADS;
+            if (t >= n) continue;
+            if (!TO_PADDED) {
+                *reinterpret_cast<C*>(dst + dense0 + (long long)t * V) = v[q];
+                continue;
+            }
+            int j, c;
+            T* o = dst + place(t, j, c);
+            auto put = [&](T* p) {   // the chunk and its images in x
+                *reinterpret_cast<C*>(p) = v[q];
+                if (c < gc) *reinterpret_cast<C*>(p + g.nx) = v[q];
+                if (c >= nc - gc) *reinterpret_cast<C*>(p - g.nx) = v[q];
+            };
+            put(o);
+            if (j < PY || j >= g.ny - PY)
+                for (int m = -PY; m <= PY; ++m) {
+                    const int jj = j + m * g.ny;
+                    if (m != 0 && jj >= -PY && jj < g.ny + PY) put(o + (long long)m * g.ny * g.nxp);
+                }
+        }
+    }
+}
+
+template <typename T, bool TO_PADDED>
+static void launch_layout(const Geom& g, const T* const src[6], T* const dst[6], int n,
+                          cudaStream_t st) {
+    constexpr int V = 16 / sizeof(T);
+    if (n <= 0) return;
+    CopyList<T> list;
+    bool wide = true;   // the padded arrays are aligned; the dense ones are the caller's
+    for (int i = 0; i < n; ++i) {
+        list.src[i] = src[i];
+        list.dst[i] = dst[i];
+        const void* dense = TO_PADDED ? (const void*)src[i] : (const void*)dst[i];
+        wide = wide && reinterpret_cast<uintptr_t>(dense) % 16 == 0;
+    }
+    const long long rows = (long long)g.ny * g.nz;
+    const int nc = g.nx / (wide ? V : 1);
+    const int R = nc < COPY_THREADS * COPY_ILP ? COPY_THREADS * COPY_ILP / nc : 1;
+    const dim3 grd((unsigned)((rows + R - 1) / R), (unsigned)n);
+    if (wide) layout_kernel<T, V, TO_PADDED><<<grd, COPY_THREADS, 0, st>>>(g, list, R);
+    else layout_kernel<T, 1, TO_PADDED><<<grd, COPY_THREADS, 0, st>>>(g, list, R);
 }
 
 template <typename T>
-__global__ void pack_kernel(Geom g, const T* __restrict__ padded, T* __restrict__ dense) {
-    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const long long n = (long long)g.nx * g.ny * g.nz;
-    if (t >= n) return;
-    const int i = (int)(t % g.nx);
-    const long long r = t / g.nx;
-    const int j = (int)(r % g.ny);
-    const int k = (int)(r / g.ny);
-    dense[t] = padded[pidx(g, i, j, k)];
-}
-
-template <typename T>
-void launch_unpack(const Geom& g, const T* dense, T* padded, cudaStream_t st) {
-    unpack_kernel<T><<<(unsigned)((g.total + 255) / 256), 256, 0, st>>>(g, dense, padded);
+void launch_unpack(const Geom& g, const T* const dense[6], T* const padded[6], int n,
+                   cudaStream_t st) {
+    launch_layout<T, true>(g, dense, padded, n, st);
 }
 template <typename T>
-void launch_pack(const Geom& g, const T* padded, T* dense, cudaStream_t st) {
-    const long long n = (long long)g.nx * g.ny * g.nz;
-    pack_kernel<T><<<(unsigned)((n + 255) / 256), 256, 0, st>>>(g, padded, dense);
+void launch_pack(const Geom& g, const T* const padded[6], T* const dense[6], int n,
+                 cudaStream_t st) {
+    launch_layout<T, false>(g, padded, dense, n, st);
 }
 // Periodic images only: every ghost cell of the padded array (rows 0 .. PY-1 and
 // ny+PY .. nyp-1, columns 0 .. PX-1 and nx+PX .. nxp-1 of the owned rows) takes the value of the
@@ -413,10 +491,14 @@ void launch_fill_ghosts(const Geom& g, T* padded, cudaStream_t st) {
 }
 template void launch_fill_ghosts<float>(const Geom&, float*, cudaStream_t);
 template void launch_fill_ghosts<double>(const Geom&, double*, cudaStream_t);
-template void launch_unpack<float>(const Geom&, const float*, float*, cudaStream_t);
-template void launch_unpack<double>(const Geom&, const double*, double*, cudaStream_t);
-template void launch_pack<float>(const Geom&, const float*, float*, cudaStream_t);
-template void launch_pack<double>(const Geom&, const double*, double*, cudaStream_t);
+template void launch_unpack<float>(const Geom&, const float* const[6], float* const[6], int,
+                                   cudaStream_t);
+template void launch_unpack<double>(const Geom&, const double* const[6], double* const[6], int,
+                                    cudaStream_t);
+template void launch_pack<float>(const Geom&, const float* const[6], float* const[6], int,
+                                 cudaStream_t);
+template void launch_pack<double>(const Geom&, const double* const[6], double* const[6], int,
+                                  cudaStream_t);
 
 // ---------------------------------------------------------------------------
 // probe: loss += sum_{j,k} (F[x_p, j, k] - T[k][j])^2   (one block: fixed summation order)

@@ -78,3 +78,40 @@ def test_plane_wave_of_denormals_and_non_finite_values():
         else:
             assert math.isnan(re) if math.isnan(ref) else re == ref
     sm.close()
+
+
+@pytest.mark.parametrize("offset", [0, 1])
+@pytest.mark.parametrize("dtype", ["f32", "f64"])
+@pytest.mark.parametrize("shape,dims", [((4, 1, 1), 1), ((8, 3, 1), 2), ((260, 5, 7), 3), ((68, 130, 9), 3)])
+def test_state_round_trip_is_exact(shape, dims, dtype, offset):
+    """set_state / get_state through the padded layout, dense arrays that start on a 16-byte boundary
+    and one element past it, a NULL component; one step after it equals the step from host memory
+    (whose images come from another kernel)."""
+    nx, ny, nz = shape
+    tt = torch.float32 if dtype == "f32" else torch.float64
+    f = [torch.from_numpy(a).to(tt) for a in _random_state(shape, dtype, 5)]
+    f[3] = None
+    dev = []
+    for a in f:
+        if a is None:
+            dev.append(None)
+            continue
+        buf = torch.empty(a.numel() + offset, dtype=tt, device="cuda")[offset:].view(a.shape)
+        buf.copy_(a)
+        dev.append(buf)
+    sm, ref = _sim(shape, dtype, dims), _sim(shape, dtype, dims)
+    sm.set_state(dev)
+    out = [torch.full((nx * ny * nz + offset,), 7.0, dtype=tt, device="cuda")[offset:].view(nz, ny, nx)
+           for _ in range(6)]
+    from paper_1710_06829_gb300 import _lib as L
+    L.fdtd_get_state(sm.h, [t.data_ptr() for t in out], L.FDTD_MEM_DEVICE)
+    torch.cuda.synchronize()
+    for a, b in zip(f, out):
+        assert torch.equal(b.cpu(), torch.zeros_like(b, device="cpu") if a is None else a)
+    ref.set_state_host(f)
+    sm.step(1)
+    ref.step(1)
+    for a, b in zip(sm.get_state(), ref.get_state()):
+        assert torch.equal(a, b)
+    sm.close()
+    ref.close()
