@@ -44,7 +44,7 @@ size_t group_scratch_doubles(const int N[3], long long npts);
 void launch_disp_group_norm(const double alpha[3], const double beta[3][3], const double delta[3],
                             double dt, const double dx[3], int dims, const int N[3], int weight,
                             double wparam, double* scratch, double** out_dev, cudaStream_t st);
-size_t norm_scratch_doubles(const int N[3], long long npts);
+size_t norm_scratch_doubles(const int N[3]);
 size_t diag_scratch_bytes(const Geom& g);
 void launch_omega(const double alpha[3], const double beta[3][3], const double delta[3], double dt,
                   const double dx[3], int dims, const double* k_dev, int n, double* out_dev,
@@ -1324,6 +1324,69 @@ void fdtd_destroy(fdtd_handle* h) {
     delete h;
 }
 
+namespace {
+
+// Scratch of one norm evaluation: one of four static areas of 256 KB on the current device, held
+// for the length of the call (which ends with a stream synchronisation), or stream-ordered memory
+// when the areas are all in use or too small.  A stream-ordered allocation a call cost 200 us: the
+// device's default pool gives its memory back at every synchronisation.  The areas live as long as
+// the module; they hold nothing between calls.
+constexpr int kNormAreas = 4, kNormDevices = 64;
+constexpr size_t kNormAreaDoubles = 32 * 1024;
+static __device__ __align__(256) double g_norm_areas[kNormAreas * kNormAreaDoubles];
+
+class NormScratch {
+public:
+    NormScratch(size_t doubles, cudaStream_t st) : st_(st) {
+        if (doubles <= kNormAreaDoubles && cudaGetDevice(&dev_) == cudaSuccess && dev_ >= 0 &&
+            dev_ < kNormDevices) {
+            void* base = nullptr;
+            if (cudaGetSymbolAddress(&base, g_norm_areas) == cudaSuccess && base) {
+                std::lock_guard<std::mutex> lock(mutex());
+                for (int i = 0; i < kNormAreas && area_ < 0; ++i)
+                    if (!busy()[dev_][i]) area_ = i;
+                if (area_ >= 0) {
+                    busy()[dev_][area_] = true;
+                    ptr = (double*)base + area_ * kNormAreaDoubles;
+                }
+            } else {
+                (void)cudaGetLastError();
+            }
+        }
+        if (!ptr) err = cudaMallocAsync((void**)&ptr, doubles * sizeof(double), st);
+    }
+    // stream-ordered memory is given back before the call's synchronisation, an area after it
+    void launched() {
+        if (ptr && area_ < 0) cudaFreeAsync(ptr, st_);
+        if (area_ < 0) ptr = nullptr;
+    }
+    ~NormScratch() {
+        launched();
+        if (area_ >= 0) {
+            std::lock_guard<std::mutex> lock(mutex());
+            busy()[dev_][area_] = false;
+        }
+    }
+    NormScratch(const NormScratch&) = delete;
+    NormScratch& operator=(const NormScratch&) = delete;
+    double* ptr = nullptr;
+    cudaError_t err = cudaSuccess;
+
+private:
+    static std::mutex& mutex() {
+        static std::mutex m;
+        return m;
+    }
+    static bool (*busy())[kNormAreas] {
+        static bool b[kNormDevices][kNormAreas] = {};
+        return b;
+    }
+    cudaStream_t st_;
+    int dev_ = -1, area_ = -1;
+};
+
+}  // namespace
+
 int disp_norm_eval(const fdtd_coeffs* coeffs, double dt, const double dx[3], int32_t dims,
                    const int32_t N[3], int32_t weight, double weight_param, double* out,
                    void* stream) {
@@ -1344,20 +1407,16 @@ int disp_norm_eval(const fdtd_coeffs* coeffs, double dt, const double dx[3], int
     if (rc) return rc;
     cudaStream_t st = (cudaStream_t)stream;
     int Nd[3];
-    long long npts = 1;
-    for (int i = 0; i < 3; ++i) {
-        Nd[i] = i < dims ? N[i] : 1;
-        npts *= Nd[i];
-    }
-    const size_t nscr = norm_scratch_doubles(Nd, npts);
-    double* scratch = nullptr;
-    CK(cudaMallocAsync((void**)&scratch, nscr * sizeof(double), st));
+    for (int i = 0; i < 3; ++i) Nd[i] = i < dims ? N[i] : 1;
+    const size_t nscr = norm_scratch_doubles(Nd);
+    NormScratch scratch(nscr, st);
+    CK(scratch.err);
     double* res = nullptr;
-    launch_disp_norm(cc.alpha, cc.beta, cc.delta, dt, dx, dims, Nd, weight, weight_param, scratch,
-                     &res, st);
+    launch_disp_norm(cc.alpha, cc.beta, cc.delta, dt, dx, dims, Nd, weight, weight_param,
+                     scratch.ptr, &res, st);
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaMemcpyAsync(out, res, 14 * sizeof(double), cudaMemcpyDeviceToHost, st);
-    cudaFreeAsync(scratch, st);
+    scratch.launched();
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) {
         set_error("disp_norm_eval: %s", cudaGetErrorString(e));
@@ -1393,14 +1452,14 @@ int disp_group_norm_eval(const fdtd_coeffs* coeffs, double dt, const double dx[3
         npts *= Nd[i];
     }
     const size_t nscr = group_scratch_doubles(Nd, npts);
-    double* scratch = nullptr;
-    CK(cudaMallocAsync((void**)&scratch, nscr * sizeof(double), st));
+    NormScratch scratch(nscr, st);
+    CK(scratch.err);
     double* res = nullptr;
     launch_disp_group_norm(cc.alpha, cc.beta, cc.delta, dt, dx, dims, Nd, weight, weight_param,
-                           scratch, &res, st);
+                           scratch.ptr, &res, st);
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaMemcpyAsync(out, res, 14 * sizeof(double), cudaMemcpyDeviceToHost, st);
-    cudaFreeAsync(scratch, st);
+    scratch.launched();
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) {
         set_error("disp_group_norm_eval: %s", cudaGetErrorString(e));
@@ -1545,12 +1604,8 @@ int disp_norm_eval_noalloc(const fdtd_coeffs* coeffs, double dt, const double dx
     int rc = validate(cc, dx, dims, dt);
     if (rc) return rc;
     int Nd[3];
-    long long npts = 1;
-    for (int i = 0; i < 3; ++i) {
-        Nd[i] = i < dims ? N[i] : 1;
-        npts *= Nd[i];
-    }
-    if (norm_scratch_doubles(Nd, npts) > kNoallocDoubles) {
+    for (int i = 0; i < 3; ++i) Nd[i] = i < dims ? N[i] : 1;
+    if (norm_scratch_doubles(Nd) > kNoallocDoubles) {
         set_error("disp_norm_eval_noalloc: grid needs more than the %zu-double static scratch",
                   kNoallocDoubles);
         return FDTD_EINVAL;

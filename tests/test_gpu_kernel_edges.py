@@ -115,3 +115,54 @@ def test_state_round_trip_is_exact(shape, dims, dtype, offset):
         assert torch.equal(a, b)
     sm.close()
     ref.close()
+
+
+# one point, segments shorter than the minimum, a ragged last segment, rows that do not fill a
+# block, empty rows under the cone, dt^2 S near 1 at the last points
+NORM_CASES = [(1, (3, 1, 1), 0.9), (1, (4096, 1, 1), 0.9999), (2, (1, 7, 1), 0.9), (2, (67, 5, 1), 0.9),
+              (2, (130, 129, 1), 0.9999), (3, (33, 2, 70), 0.95), (3, (70, 64, 3), 0.95)]
+
+
+@pytest.mark.parametrize("weight,par", [(0, 0.0), (1, math.radians(30)), (1, math.radians(3)),
+                                        (1, math.radians(120)), (2, 0.1)])
+@pytest.mark.parametrize("dims,N,courant", NORM_CASES)
+def test_norm_segments_and_weights_match_oracle(dims, N, courant, weight, par):
+    """Row segments, cone starts and the angle table.  omega has a relative error of a few eps
+    divided by sqrt(1 - dt^2 S), as in the plain formulas; rel 1e-11 covers it."""
+    from oracle import dispersion as D
+    from paper_1710_06829_gb300 import inputs
+    from paper_1710_06829_gb300 import sim as S
+    beta, delta = np.zeros((3, 3)), np.zeros(3)
+    if dims > 1:
+        beta, delta = inputs.isotropic_theta(-0.05, -0.04, 0.02, 0.01)
+    dx = [1.0, 1.2, 0.9]
+    dt = courant * D.dt_max(beta, delta, dx, dims)
+    f, gb, gd, gdt = S.disp_norm(beta, delta, dt, dx, dims, N, weight, par)
+    kind = (D.WEIGHT_UNIFORM, D.WEIGHT_CONE_X, D.WEIGHT_GAUSS_Y)[weight]
+    rf, rgb, rgd, rgdt = D.norm_and_grad(beta, delta, dt, dx, N, dims, kind, par)
+    got = np.r_[f, np.ravel(gb), gd, gdt]
+    ref = np.r_[rf, np.ravel(rgb), rgd, rgdt]
+    assert np.all(np.abs(got - ref) <= 1e-11 * np.abs(ref) + 1e-13 * max(1.0, abs(rf)))
+
+
+def test_norm_from_several_threads_and_streams():
+    """More concurrent evaluations than scratch areas: every one returns its own value."""
+    import threading
+
+    from paper_1710_06829_gb300 import sim as S
+    beta, delta = np.zeros((3, 3)), np.zeros(3)
+    args = [(0.3 + 0.02 * i, [1.0, 1.0, 1.0], 2, (200 + i, 150, 1)) for i in range(8)]
+    ref = [S.disp_norm(beta, delta, *a)[0] for a in args]
+    bad = []
+
+    def work(i):
+        st = torch.cuda.Stream()
+        for _ in range(20):
+            if S.disp_norm(beta, delta, *args[i], stream=st)[0] != ref[i]:
+                bad.append(i)
+    th = [threading.Thread(target=work, args=(i,)) for i in range(len(args))]
+    for t in th:
+        t.start()
+    for t in th:
+        t.join()
+    assert not bad
