@@ -271,7 +271,7 @@ static int adjoint32_tz(const Geom& g) {
     static int slots = -1;
     if (slots < 0) slots = resident_slots((const void*)adj32::adjB_kernel, adj32::NT, adj32::SMEM);
     // shorter chunks suit this kernel: at 256^3, 19 planes 0.37 ms, 26: 0.38, 37: 0.42
-    return zchunk_len((g.nx / adj32::TX) * (g.ny / adj32::TY), g.nz, slots, 16, 24);
+    return zchunk_waves((g.nx / adj32::TX) * (g.ny / adj32::TY), g.nz, slots, 16, 24);
 }
 
 int adjoint32_blocks(const Geom& g) {

@@ -286,7 +286,7 @@ bool adjoint32e_prepare() {
 static int adjoint32e_tz(const Geom& g) {
     static int slots = -1;
     if (slots < 0) slots = resident_slots((const void*)adj32e::adjE_kernel, adj32e::NT, adj32e::SMEM);
-    return zchunk_len((g.nx / adj32e::TX) * (g.ny / adj32e::TY), g.nz, slots, 16, 64);
+    return zchunk_waves((g.nx / adj32e::TX) * (g.ny / adj32e::TY), g.nz, slots, 16, 64);
 }
 
 // maps.e[c]: 72 x 12 boxes of mu_c (= lambda_B component c after the adjoint B half)

@@ -622,12 +622,15 @@ bool adjoint32f_prepare() {
                                 (int)adj32f::SMEM) == cudaSuccess;
 }
 
+// Chunk length in [16, 64] with the fewest waves x (planes + 2).  A chunk's planes are one
+// compensated FP32 sum per thread, so the rule also fixes the gradient's rounding: it is kept as it
+// is (another split moves the gradient by some 1e-9), unlike the forward step's.
 static int adjoint32f_tz(const Geom& g) {
     static int slots = -1;
     if (slots < 0)
         slots = resident_slots_tmem((const void*)adj32f::adjF_kernel<true>, adj32f::NT, adj32f::SMEM,
                                     adj32f::TM_COLS);
-    return zchunk_len((g.nx / adj32f::TX) * (g.ny / adj32f::TY), g.nz, slots, 16, 64);
+    return zchunk_waves((g.nx / adj32f::TX) * (g.ny / adj32f::TY), g.nz, slots, 16, 64);
 }
 
 int adjoint32f_blocks(const Geom& g) {

@@ -1,7 +1,7 @@
 // FP32 fused leapfrog step (one launch per leapfrog step).
 //
 // A CTA owns a 64 x 8 (x, y) tile and a chunk of tz planes (a launch parameter) and marches
-// through it.  E^n planes arrive by TMA (cp.async.bulk.tensor.3d) as 76 x 12 boxes (x0-4 ..,
+// through it; the last tiles of a ragged grid reach past its cells and drop what they form there.  E^n planes arrive by TMA (cp.async.bulk.tensor.3d) as 76 x 12 boxes (x0-4 ..,
 // y0-2 ..) into a ring of five shared-memory slots, one plane ahead of use, completion signalled
 // on mbarriers.  Iteration `it` forms B^{n+1/2} on plane p = z0-1+it (tile, halo row y0-1, halo
 // column x0-1) and E^{n+1} on plane p-1, so one block barrier per plane suffices; B^{n+1/2}
@@ -119,7 +119,7 @@ step_kernel(const __grid_constant__ FusedMaps maps, Geom g, Mult<float> m, Mult2
     float* sB = reinterpret_cast<float*>(smem + OFF_BN);
     uint64_t* bar = reinterpret_cast<uint64_t*>(smem + OFF_BAR);
 
-    const int ntx = g.nx / TX, nty = g.ny / TY;
+    const int ntx = (g.nx + TX - 1) / TX, nty = (g.ny + TY - 1) / TY;
     int w = blockIdx.x;
     const int tx = w % ntx;
     w /= ntx;
@@ -174,12 +174,16 @@ step_kernel(const __grid_constant__ FusedMaps maps, Geom g, Mult<float> m, Mult2
     const bool rb = b_bx < 0 || b_bx == TX - W;
     const int e = (b_by + 2) * EW + (b_bx + 4);   // in-plane index of the segment, E box
     const int bi = (b_by + 1) * BW + (b_bx + 4);  // in-plane index of the segment, B ring
-    const unsigned b_off = (unsigned)((y0 + b_by + PY) * g.nxp + (x0 + b_bx + PX));
+    // the last tiles of a ragged grid reach past its cells: segments at i >= nx or j >= ny compute
+    // on what the boxes hold there (ghosts, then zeros) and drop the results; their global reads
+    // are moved back onto the last segment
+    const bool live = x0 + b_bx < g.nx && y0 + b_by < g.ny;
+    const int b_i = min(x0 + b_bx, g.nx - W), b_j = min(y0 + b_by, g.ny - 1);
+    const unsigned b_off = (unsigned)((b_j + PY) * g.nxp + (b_i + PX));
     const unsigned plane = (unsigned)g.plane;
-    int b_y = y0 + b_by;
-    if (b_y < 0) b_y += g.ny;
+    const int b_y = b_j < 0 ? b_j + g.ny : b_j;
     // owned-cell destinations of this thread's segment
-    const SegOut dst = seg_out(g, x0 + (b_bx < 0 ? 0 : b_bx), y0 + (b_by < 0 ? 0 : b_by), edge);
+    const SegOut dst = seg_out(g, max(b_i, 0), max(b_j, 0), edge);
 
     if (tid == PRODUCER) {
         for (int s = 0; s <= NS; ++s) mbar_init(&bar[s], 1);
@@ -392,7 +396,7 @@ step_kernel(const __grid_constant__ FusedMaps maps, Geom g, Mult<float> m, Mult2
                 tm_st(tb + COL_BY + 4 * e3, byv);
                 tm_st(tb + COL_BZ + 4 * (it & 1), bzv);
             }
-            if (p >= z0 && b_own) {
+            if (p >= z0 && b_own && live) {
                 const unsigned po = (unsigned)pw * plane;
                 put_seg(out.c[3], po, dst, bxv);
                 put_seg(out.c[4], po, dst, byv);
@@ -455,7 +459,7 @@ step_kernel(const __grid_constant__ FusedMaps maps, Geom g, Mult<float> m, Mult2
                 upk(ry, ey[u], ey[u + 1]);
                 upk(rz, ez[u], ez[u + 1]);
             }
-            const int i0 = x0 + b_bx, j = y0 + b_by;
+            const int i0 = b_i, j = b_j;
             if (jx_row != nullptr) {
                 float jv[W];
                 unpackv(__ldg(reinterpret_cast<const float4*>(jx_row + i0)), jv);
@@ -468,14 +472,16 @@ step_kernel(const __grid_constant__ FusedMaps maps, Geom g, Mult<float> m, Mult2
 #pragma unroll
                 for (int u = 0; u < W; ++u) { ex[u] *= f; ey[u] *= f; ez[u] *= f; }
             }
-#pragma unroll
-            for (int u = 0; u < W; ++u)
-                fin = nonfinite_acc(nonfinite_acc(nonfinite_acc(fin, ex[u]), ey[u]), ez[u]);
             const unsigned po = (unsigned)qw * plane;
-            put_seg(out.c[0], po, dst, ex);
-            put_seg(out.c[1], po, dst, ey);
-            put_seg(out.c[2], po, dst, ez);
-            if (h0 != nullptr) {
+            if (live) {
+#pragma unroll
+                for (int u = 0; u < W; ++u)
+                    fin = nonfinite_acc(nonfinite_acc(nonfinite_acc(fin, ex[u]), ey[u]), ez[u]);
+                put_seg(out.c[0], po, dst, ex);
+                put_seg(out.c[1], po, dst, ey);
+                put_seg(out.c[2], po, dst, ez);
+            }
+            if (h0 != nullptr && live) {
                 put_seg(h0, po, dst, ex);
                 put_seg(h1, po, dst, ey);
                 put_seg(h2, po, dst, ez);
@@ -519,10 +525,23 @@ step_kernel(const __grid_constant__ FusedMaps maps, Geom g, Mult<float> m, Mult2
 
 }  // namespace f32seg
 
+static int tiles32(const Geom& g) {
+    using namespace f32seg;
+    return ((g.nx + TX - 1) / TX) * ((g.ny + TY - 1) / TY);
+}
+
+// The kernel handles any nx >= 8 (a multiple of 4) and ny >= 4: below, a cell has images on both
+// sides and put_seg's single offsets do not cover them.  A tile that reaches past the grid does
+// idle work, but even where most of it is idle the kernel is the faster one (us a step, this kernel
+// and the two reference-form kernels: 300 x 250 x 112 109 / 225, 132 x 130 x 200 65 / 109,
+// 16 x 300 x 300 66 / 111, 32^3 8.6 / 10.7, 68 x 9 x 64 10.6 / 10.5).
+// Ragged grids of fewer than four planes stay with the reference form: the march forms two B
+// planes and reads five E planes for each chunk's first one (1000 x 750 x 1: 27 us against 24).
 bool fused32_supported(const Geom& g) {
-    // 32-bit element offsets inside the kernel
-    return g.nx % f32seg::TX == 0 && g.ny % f32seg::TY == 0 && g.nx >= f32seg::TX &&
-           g.ny >= f32seg::TY && g.total < (1LL << 31);
+    using namespace f32seg;
+    const bool whole = g.nx % TX == 0 && g.ny % TY == 0;
+    return g.nx >= 2 * PX && g.ny >= 2 * PY && (whole || g.nz >= 4) &&
+           g.total < (1LL << 31);   // 32-bit element offsets
 }
 
 int fused32_ebox_w() { return f32seg::EW; }
@@ -570,10 +589,32 @@ int resident_slots_tmem(const void* kernel, int threads, size_t smem, int tmem_c
     return n > 0 ? sms * n : 0;
 }
 
-int zchunk_len(int tiles_xy, int nz, int slots, int tz_min, int tz_max) {
-    // A CTA marches tz planes plus about two planes of fixed cost (the z-halo B plane and the
-    // prologue copies); CTAs run in waves of `slots`.  Minimise waves x (tz + 2) over chunk
-    // lengths tz_min..tz_max; ties go to the longer chunk.
+int zchunk_len(int tiles_xy, int nz, int slots, int fixed, int tz_max) {
+    // A CTA marches tz planes plus `fixed` planes' worth of prologue (halo planes, first copies); the
+    // CTAs start in order (tiles fastest, the short last chunk last) as slots come free.  The chunk
+    // length with the shortest schedule wins, ties go to the longer chunk.  A grid that does not
+    // fill the device thus gets short chunks: 64^3 took 35.2 us a step in chunks of 16 planes (the
+    // former least length), 12.6 us in chunks of 2; 128^3 39.4 -> 33.2 us in chunks of 10.
+    const int hi = nz < tz_max ? nz : tz_max;
+    if (slots <= 0) return hi;
+    int best = hi;
+    long long best_cost = -1;
+    for (int tz = hi; tz >= 1; --tz) {
+        const int chunks = (nz + tz - 1) / tz;
+        const long long a = tz + fixed, b = nz - (long long)(chunks - 1) * tz + fixed;
+        const long long full = (long long)tiles_xy * (chunks - 1);
+        const long long waves = full / slots, busy = full % slots, free = slots - busy;
+        const long long tail = (tiles_xy + free - 1) / free * b;   // the last chunk's CTAs
+        const long long cost = waves * a + (busy > 0 && a > tail ? a : tail);
+        if (best_cost < 0 || cost < best_cost) {
+            best_cost = cost;
+            best = tz;
+        }
+    }
+    return best;
+}
+
+int zchunk_waves(int tiles_xy, int nz, int slots, int tz_min, int tz_max) {
     const int hi = nz < tz_max ? nz : tz_max;
     if (slots <= 0) return hi;
     int best = hi;
@@ -581,7 +622,7 @@ int zchunk_len(int tiles_xy, int nz, int slots, int tz_min, int tz_max) {
     for (int tz = hi; tz >= tz_min || tz == nz; --tz) {
         const long long ctas = (long long)tiles_xy * ((nz + tz - 1) / tz);
         const long long waves = (ctas + slots - 1) / slots;
-        const long long cost = waves * (tz + 2);
+        const long long cost = waves * (tz + 2);   // ties go to the longer chunk
         if (best_cost < 0 || cost < best_cost) {
             best_cost = cost;
             best = tz;
@@ -597,7 +638,7 @@ static int fused32_tz(const Geom& g) {
     if (slots < 0) slots = resident_slots_tmem((const void*)step_kernel, NT, SMEM, TM_COLS);
     // measured at 256^3 (456 resident CTAs): 37-plane chunks (2 full waves) 0.218 ms per step,
     // 32-plane chunks (2.25 waves) 0.269 ms
-    return zchunk_len((g.nx / TX) * (g.ny / TY), g.nz, slots, 16, 64);
+    return zchunk_len(tiles32(g), g.nz, slots, 2, 64);
 }
 
 void launch_fused32(const FusedMaps& maps, FieldSet<float> in, const Geom& g, const Mult<float>& m,
@@ -605,7 +646,7 @@ void launch_fused32(const FusedMaps& maps, FieldSet<float> in, const Geom& g, co
                     const float* jx_row, float* hist_E[3], int* err, cudaStream_t st) {
     using namespace f32seg;
     const int tz = fused32_tz(g);
-    const int nblk = (g.nx / TX) * (g.ny / TY) * ((g.nz + tz - 1) / tz);
+    const int nblk = tiles32(g) * ((g.nz + tz - 1) / tz);
     step_kernel<<<nblk, NT, SMEM, st>>>(maps, g, m, make_mult2(m), in, out, spy, spz, jyz, jx_row, hist_E[0],
                                         hist_E[1], hist_E[2], 0, g.nz, tz, err);
 }
@@ -619,7 +660,7 @@ void launch_fused32_range(const FusedMaps& maps, FieldSet<float> in, const Geom&
     using namespace f32seg;
     static int slots = -1;
     if (slots < 0) slots = resident_slots_tmem((const void*)step_kernel, NT, SMEM, TM_COLS);
-    const int tiles = (g.nx / TX) * (g.ny / TY);
+    const int tiles = tiles32(g);
     const int len = ze - zs;
     const int tz = zchunk_len(tiles, len, slots, 2, 64);
     const int nblk = tiles * ((len + tz - 1) / tz);

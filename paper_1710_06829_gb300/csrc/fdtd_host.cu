@@ -708,7 +708,9 @@ static int ensure_hist(fdtd_handle* h, int snaps) {
     const size_t arr = (size_t)h->g.total * h->esz;
     CK(cudaMalloc(&h->hist, (size_t)snaps * 3 * arr));
     h->hist_cap = snaps;
-    if (h->grid.dtype == FDTD_F32 && h->plan && adjoint32_supported(h->g) && adjoint32_prepare()) {
+    // the two-kernel reverse step reads E^n through descriptors (the one-kernel step does not)
+    if (h->grid.dtype == FDTD_F32 && h->plan && h->adj_split && adjoint32_supported(h->g) &&
+        adjoint32_prepare()) {
         h->hist_maps.resize(snaps);
         for (int s = 0; s < snaps; ++s)
             for (int c = 0; c < 3; ++c)
@@ -965,7 +967,7 @@ static int adjoint_impl(fdtd_handle* h, int n, const fdtd_probe* probe, double* 
     int rc = ensure_lam(h);
     if (rc) return rc;
     const bool staged = std::is_same<T, float>::value && !h->hist_maps.empty();
-    const bool one_kernel = staged && h->lam_fused;
+    const bool one_kernel = std::is_same<T, float>::value && h->lam_fused;
     const int nblk = one_kernel ? adjoint32f_blocks(g) : staged ? adjoint32_blocks(g) : adjoint_B_blocks(g);
     if (h->npart < nblk) {
         if (h->partials) cudaFree(h->partials);

@@ -171,13 +171,15 @@ void launch_reduce_grad(const double* part, int nblocks, GradScale sc, double* g
                         cudaStream_t st);
 
 // Resident CTAs of `kernel` on the whole device (SMs x CTAs per SM; 0 if unknown), and the
-// z-chunk length in [tz_min, tz_max] of a tiled plane-marching kernel with `tiles_xy` CTAs per
-// z-chunk that fills whole waves of `slots` CTAs best.
+// z-chunk length up to tz_max of a tiled plane-marching kernel with `tiles_xy` CTAs per z-chunk,
+// each with a prologue worth `fixed` planes, that `slots` resident CTAs finish first.
 int resident_slots(const void* kernel, int threads, size_t smem);
 // the same for a kernel that allocates tmem_cols TMEM columns per CTA (the occupancy API
 // under-reports those)
 int resident_slots_tmem(const void* kernel, int threads, size_t smem, int tmem_cols);
-int zchunk_len(int tiles_xy, int nz, int slots, int tz_min, int tz_max);
+int zchunk_len(int tiles_xy, int nz, int slots, int fixed, int tz_max);
+// the reverse steps' rule: fewest waves x (tz + 2) over tz_min .. tz_max
+int zchunk_waves(int tiles_xy, int nz, int slots, int tz_min, int tz_max);
 
 // thread-local error message
 void set_error(const char* fmt, ...);

@@ -166,3 +166,37 @@ def test_norm_from_several_threads_and_streams():
     for t in th:
         t.join()
     assert not bad
+
+
+def _step_pair(shape, dtype, monkeypatch, steps=5, dims=3, **kw):
+    """The state after `steps` steps with the tiled and with the reference-form kernels."""
+    from paper_1710_06829_gb300 import sim as S
+    f = [torch.from_numpy(a) for a in _random_state(shape, dtype, 11)]
+    out = []
+    for flag in ("1", "0"):
+        monkeypatch.setenv("FDTD_FUSED", flag)
+        sm = _sim(shape, dtype, dims, **kw)
+        sm.set_state(f)
+        src = None
+        if dims == 3 and not kw.get("batched"):
+            src = S.Bunch(1.0, 0.9, 3.0, 2.0, 1.0, 2.0, 2.0)
+        sm.step(steps, source=src)
+        sm.sync()
+        out.append(sm.get_state())
+        sm.close()
+    return out
+
+
+# narrowest grids, last tiles of one column group or one row, ghosts of the last cells in the same
+# and in a further tile, the fewest planes, more planes than a z-chunk
+RAGGED = [(8, 4, 4), (60, 12, 5), (64, 9, 4), (68, 8, 7), (132, 31, 4), (124, 30, 40), (300, 20, 70)]
+
+
+@pytest.mark.parametrize("sponge", [False, True])
+@pytest.mark.parametrize("shape", RAGGED)
+def test_ragged_tiles_step_bitwise_like_the_reference_form(shape, sponge, monkeypatch):
+    if sponge and min(shape[1:]) < 4:
+        pytest.skip("no room for the layers")
+    kw = dict(absorb_cells=2, absorb_sigma=0.3) if sponge else {}
+    for a, b in zip(*_step_pair(shape, "f32", monkeypatch, **kw)):
+        assert torch.equal(a, b)
