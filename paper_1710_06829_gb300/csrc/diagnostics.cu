@@ -30,8 +30,9 @@ int diag_blocks(const Geom& g) {
 
 // Block sums of v into part, then the grid's sums by the block that arrives last (`ticket` counts
 // the blocks and is left at zero for the next launch): always the same order, whichever block it
-// is, and no second launch (a one-block summing kernel took 5.6 us after each diagnostic).
-template <int NV>
+// is, and no second launch (a one-block summing kernel took 5.6 us after each diagnostic).  ADD:
+// out += the sums.
+template <int NV, bool ADD = false>
 __device__ __forceinline__ void reduce_finish(double (&v)[NV], double* __restrict__ part,
                                               unsigned* __restrict__ ticket, double scale,
                                               double* __restrict__ out) {
@@ -68,7 +69,7 @@ __device__ __forceinline__ void reduce_finish(double (&v)[NV], double* __restric
 #pragma unroll
         for (int q = 0; q < NV; ++q) t[q] += __ldcg(part + (long long)b * NV + q);
     const double total = block_sum(t);
-    if (threadIdx.x < NV) out[threadIdx.x] = scale * total;
+    if (threadIdx.x < NV) out[threadIdx.x] = (ADD ? out[threadIdx.x] : 0.0) + scale * total;
     if (threadIdx.x == 0) *ticket = 0;
 }
 
@@ -95,6 +96,25 @@ energy_kernel(Geom g, FieldSet<T> s, int x_lo, int x_len, int my, int mz, double
         }
     }
     reduce_finish<1>(acc, part, ticket, scale, out);
+}
+
+// loss += sum_{j,k} (F[x_p, j, k] - T[k][j])^2.  Every value of the plane lies in a sector of its
+// own, so the kernel is bound by their latency: one value a thread over as many blocks as that
+// gives (up to the scratch's) keeps them all in flight.  128 x 128 values: 22.4 us in one block
+// (the former kernel), 6.1 us here.
+template <typename T>
+__global__ void __launch_bounds__(DG_THREADS)
+probe_loss_kernel(Geom g, const T* __restrict__ F, int xp, const T* __restrict__ target,
+                  double* part, unsigned* ticket, double* loss) {
+    double acc[1] = {0.0};
+    const long long n = (long long)g.ny * g.nz;
+    for (long long t = (long long)blockIdx.x * DG_THREADS + threadIdx.x; t < n;
+         t += (long long)gridDim.x * DG_THREADS) {
+        const int k = (int)(t / g.ny), j = (int)(t - (long long)k * g.ny);
+        const double d = (double)F[pidx(g, xp, j, k)] - (double)target[t];
+        acc[0] += d * d;
+    }
+    reduce_finish<1, true>(acc, part, ticket, 1.0, loss);
 }
 
 // (cos, sin) of w (m + o) for m < n: one entry per grid line of an axis
@@ -405,6 +425,18 @@ void launch_energy(const Geom& g, FieldSet<T> s, int x_lo, int x_len, int my, in
     energy_kernel<T><<<diag_blocks(g), DG_THREADS, 0, st>>>(g, s, x_lo, x_len, my, mz, d.part,
                                                             d.ticket, 0.5 * dV, out);
 }
+
+template <typename T>
+void launch_probe_loss(const Geom& g, const T* E, int x_index, const T* target, double* scratch,
+                       double* loss, cudaStream_t st) {
+    const DiagScratch d = diag_scratch(g, scratch);
+    probe_loss_kernel<T><<<blocks_of((long long)g.ny * g.nz, g), DG_THREADS, 0, st>>>(
+        g, E, x_index, target, d.part, d.ticket, loss);
+}
+template void launch_probe_loss<float>(const Geom&, const float*, int, const float*, double*,
+                                       double*, cudaStream_t);
+template void launch_probe_loss<double>(const Geom&, const double*, int, const double*, double*,
+                                        double*, cudaStream_t);
 
 template <typename T>
 void launch_planewave(const Geom& g, const T* F, const double k[3], const double off[3],

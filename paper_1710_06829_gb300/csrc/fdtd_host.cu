@@ -722,6 +722,18 @@ static int ensure_hist(fdtd_handle* h, int snaps) {
     return FDTD_OK;
 }
 
+static int ensure_dpart(fdtd_handle* h) {
+    if (h->dpart) return FDTD_OK;
+    CK(cudaMalloc(&h->dpart, diag_scratch_bytes(h->g)));
+    cudaError_t e = cudaMemsetAsync(h->dpart, 0, 16, h->stream);   // the block ticket
+    if (e != cudaSuccess) {
+        cudaFree(h->dpart);
+        h->dpart = nullptr;
+        CK(e);
+    }
+    return FDTD_OK;
+}
+
 static int ensure_jx(fdtd_handle* h, int n) {
     if (h->jx_cap >= n) return FDTD_OK;
     if (h->jx) { cudaFree(h->jx); h->jx = nullptr; h->jx_cap = 0; }
@@ -821,6 +833,10 @@ static int step_impl(fdtd_handle* h, int n, const fdtd_source* src, const fdtd_p
                               h->step, (T*)h->jx, h->stream);
         CK(cudaGetLastError());
     }
+    if (probe) {
+        int rc = ensure_dpart(h);
+        if (rc) return rc;
+    }
     if (record) {
         int rc = ensure_hist(h, n + 1);
         if (rc) return rc;
@@ -882,7 +898,7 @@ static int step_impl(fdtd_handle* h, int n, const fdtd_source* src, const fdtd_p
         if (probe) {
             const T* tgt = (const T*)probe->target + (size_t)(h->step - 1) * g.ny * g.nz;
             launch_probe_loss<T>(g, (const T*)h->arr(h->cur, probe->component), probe->x_index,
-                                 tgt, loss, h->stream);
+                                 tgt, h->dpart, loss, h->stream);
             CK(cudaGetLastError());
         }
     }
@@ -1057,18 +1073,6 @@ int fdtd_step_adjoint(fdtd_handle* h, int32_t n, const fdtd_probe* probe, double
     }
     if (h->grid.dtype == FDTD_F32) return adjoint_impl<float>(h, n, probe, grad_dev);
     return adjoint_impl<double>(h, n, probe, grad_dev);
-}
-
-static int ensure_dpart(fdtd_handle* h) {
-    if (h->dpart) return FDTD_OK;
-    CK(cudaMalloc(&h->dpart, diag_scratch_bytes(h->g)));
-    cudaError_t e = cudaMemsetAsync(h->dpart, 0, 16, h->stream);   // the block ticket
-    if (e != cudaSuccess) {
-        cudaFree(h->dpart);
-        h->dpart = nullptr;
-        CK(e);
-    }
-    return FDTD_OK;
 }
 
 int fdtd_diagnostic(fdtd_handle* h, int32_t kind, const double* params, double* out_dev) {

@@ -144,9 +144,10 @@ void launch_adjoint_E_v0(const Geom& g, const Mult<T>& m, FieldSet<T> lam, const
                          const T* sponge_z, cudaStream_t st);
 int adjoint_B_blocks(const Geom& g);
 
+// *loss += sum_{j,k} (E[x_index, j, k] - target[k][j])^2; scratch: the diagnostics' scratch
 template <typename T>
-void launch_probe_loss(const Geom& g, const T* E, int x_index, const T* target, double* loss,
-                       cudaStream_t st);
+void launch_probe_loss(const Geom& g, const T* E, int x_index, const T* target, double* scratch,
+                       double* loss, cudaStream_t st);
 template <typename T>
 void launch_probe_adjoint(const Geom& g, T* lamE, const T* E, int x_index, const T* target,
                           cudaStream_t st);

@@ -501,29 +501,8 @@ template void launch_pack<double>(const Geom&, const double* const[6], double* c
                                   cudaStream_t);
 
 // ---------------------------------------------------------------------------
-// probe: loss += sum_{j,k} (F[x_p, j, k] - T[k][j])^2   (one block: fixed summation order)
+// probe source of the reverse step (the probe's loss is with the other sums in diagnostics.cu)
 // ---------------------------------------------------------------------------
-
-template <typename T>
-__global__ void probe_loss_kernel(Geom g, const T* __restrict__ F, int xp,
-                                  const T* __restrict__ target, double* loss) {
-    double acc = 0.0;
-    const int n = g.ny * g.nz;
-    for (int t = threadIdx.x; t < n; t += blockDim.x) {
-        const int j = t % g.ny, k = t / g.ny;
-        const double d = (double)F[pidx(g, xp, j, k)] - (double)target[(long long)k * g.ny + j];
-        acc += d * d;
-    }
-    __shared__ double red[32];
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        acc = threadIdx.x < (blockDim.x >> 5) ? red[threadIdx.x] : 0.0;
-        for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
-        if (threadIdx.x == 0) *loss += acc;
-    }
-}
 
 // lambda_E[x_p, j, k] += 2 (F[x_p, j, k] - T[k][j]), written with its periodic images.
 template <typename T>
@@ -538,20 +517,11 @@ __global__ void probe_adjoint_kernel(Geom g, T* __restrict__ lam, const T* __res
 }
 
 template <typename T>
-void launch_probe_loss(const Geom& g, const T* E, int x_index, const T* target, double* loss,
-                       cudaStream_t st) {
-    probe_loss_kernel<T><<<1, 1024, 0, st>>>(g, E, x_index, target, loss);
-}
-template <typename T>
 void launch_probe_adjoint(const Geom& g, T* lamE, const T* E, int x_index, const T* target,
                           cudaStream_t st) {
     const int n = g.ny * g.nz;
     probe_adjoint_kernel<T><<<(n + 255) / 256, 256, 0, st>>>(g, lamE, E, x_index, target);
 }
-template void launch_probe_loss<float>(const Geom&, const float*, int, const float*, double*,
-                                       cudaStream_t);
-template void launch_probe_loss<double>(const Geom&, const double*, int, const double*, double*,
-                                        cudaStream_t);
 template void launch_probe_adjoint<float>(const Geom&, float*, const float*, int, const float*,
                                           cudaStream_t);
 template void launch_probe_adjoint<double>(const Geom&, double*, const double*, int,

@@ -200,3 +200,24 @@ def test_ragged_tiles_step_bitwise_like_the_reference_form(shape, sponge, monkey
     kw = dict(absorb_cells=2, absorb_sigma=0.3) if sponge else {}
     for a, b in zip(*_step_pair(shape, "f32", monkeypatch, **kw)):
         assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("dtype", ["f32", "f64"])
+@pytest.mark.parametrize("shape", [(8, 1, 1), (12, 15, 17), (64, 16, 17), (8, 700, 600)])
+def test_probe_loss_sums_the_plane(shape, dtype):
+    """One value, a ragged block, more values than threads in a wave; added to what is there.  Sums of
+    n positive terms in FP64: n eps relative, 1e-12 taken for up to 4e5."""
+    from paper_1710_06829_gb300 import sim as S
+    nx, ny, nz = shape
+    f = _random_state(shape, dtype, 21)
+    tt = torch.float32 if dtype == "f32" else torch.float64
+    tgt = torch.from_numpy(np.random.default_rng(4).standard_normal((2, nz, ny))).to(tt).cuda()
+    sm = _sim(shape, dtype, 1 if ny == 1 else 3)
+    sm.set_state([torch.from_numpy(a) for a in f])
+    loss = torch.full((1,), 3.0, dtype=torch.float64, device="cuda")
+    ref = 3.0
+    for s in range(2):
+        sm.step(1, probe=S.Probe(2, nx - 1, tgt), loss=loss)
+        ref += float(((sm.get_state()[2][:, :, nx - 1].double() - tgt[s].double()) ** 2).sum())
+    assert abs(float(loss) - ref) <= 1e-12 * ref
+    sm.close()
