@@ -268,16 +268,20 @@ static EncodeTiledFn encode_fn() {
 void launch_fused32_range(const FusedMaps& maps, FieldSet<float> in, const Geom& g,
                           const Mult<float>& m, FieldSet<float> out, const float* spy,
                           const float* spz, int zs, int ze, int* err, cudaStream_t st);
-bool fused32_supported(const Geom& g);
+bool fused32_supported(const Geom& g, bool flat);
 int fused32_ebox_w();
 bool fused32_prepare();
 void launch_fused32(const FusedMaps& maps, FieldSet<float> in, const Geom& g, const Mult<float>& m,
                     FieldSet<float> out, const float* spy, const float* spz, const float* jyz,
                     const float* jx_row, float* hist_E[3], int* err, cudaStream_t st);
 
+void launch_step2d32(const Geom& g, const Mult<float>& m, FieldSet<float> in, FieldSet<float> out,
+                     const float* spy, const float* spz, const float* jyz, const float* jx_row,
+                     float* hist_E[3], int* err, cudaStream_t st);
+
 template <typename T>
-bool fused_supported(const Geom& g) {
-    if constexpr (std::is_same<T, float>::value) return fused32_supported(g);
+bool fused_supported(const Geom& g, bool flat) {
+    if constexpr (std::is_same<T, float>::value) return fused32_supported(g, flat);
     using C = FusedCfg<T>;
     return g.nx % C::TX == 0 && g.ny % C::TY == 0 && g.nx >= C::TX && g.ny >= C::TY;
 }
@@ -308,10 +312,11 @@ bool encode_box_f32(CUtensorMap* map, const Geom& g, float* base, int bw, int bh
 }
 
 template <typename T>
-FusedPlan* fused_plan_create(const Geom& g, T* const set0[6], T* const set1[6]) {
-    if (!fused_supported<T>(g)) return nullptr;
+FusedPlan* fused_plan_create(const Geom& g, bool flat, T* const set0[6], T* const set1[6]) {
+    if (!fused_supported<T>(g, flat)) return nullptr;
     FusedPlan* p = new FusedPlan();
     p->dtype = sizeof(T) == 4 ? FDTD_F32 : FDTD_F64;
+    p->flat = flat;
     using Lc = Layout<T>;
     for (int s = 0; s < 2; ++s) {
         T* const* set = s == 0 ? set0 : set1;
@@ -388,6 +393,10 @@ void launch_step_fused(const FusedPlan* plan, int in_set, const Geom& g, const M
                        FieldSet<T> in, FieldSet<T> out, const T* sponge_y, const T* sponge_z,
                        const T* jyz, const T* jx_row, T* hist_E[3], int* err, cudaStream_t st) {
     if constexpr (std::is_same<T, float>::value) {
+        if (plan->flat) {
+            launch_step2d32(g, m, in, out, sponge_y, sponge_z, jyz, jx_row, hist_E, err, st);
+            return;
+        }
         launch_fused32(plan->maps[in_set], in, g, m, out, sponge_y, sponge_z, jyz, jx_row, hist_E,
                        err, st);
         return;
@@ -399,10 +408,10 @@ void launch_step_fused(const FusedPlan* plan, int in_set, const Geom& g, const M
         hist_E[2], err);
 }
 
-template bool fused_supported<float>(const Geom&);
-template bool fused_supported<double>(const Geom&);
-template FusedPlan* fused_plan_create<float>(const Geom&, float* const[6], float* const[6]);
-template FusedPlan* fused_plan_create<double>(const Geom&, double* const[6], double* const[6]);
+template bool fused_supported<float>(const Geom&, bool);
+template bool fused_supported<double>(const Geom&, bool);
+template FusedPlan* fused_plan_create<float>(const Geom&, bool, float* const[6], float* const[6]);
+template FusedPlan* fused_plan_create<double>(const Geom&, bool, double* const[6], double* const[6]);
 template void launch_step_fused<float>(const FusedPlan*, int, const Geom&, const Mult<float>&,
                                        FieldSet<float>, FieldSet<float>, const float*, const float*, const float*,
                                        const float*, float* [3], int*, cudaStream_t);

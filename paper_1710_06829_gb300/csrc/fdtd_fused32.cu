@@ -39,7 +39,6 @@
 // bounded (fdtd_tma.cuh); on expiry the CTA raises *err, drains its copies in flight (bounded)
 // and returns.
 #include <algorithm>
-#include <cstring>
 
 #include "fdtd_seg.cuh"
 #include "fdtd_tmem.cuh"
@@ -48,29 +47,6 @@ namespace fdtd {
 namespace f32seg {
 
 using namespace seg;
-
-// the FP32 multipliers, each duplicated into a pair for the paired arithmetic
-struct Mult2 {
-    u64 cA[3], cD[3], cB[3][3], cE[3], ncE[3];   // ncE = -cE
-};
-
-inline Mult2 make_mult2(const Mult<float>& m) {
-    auto dup = [](float v) {
-        u64 r;
-        const float two[2] = {v, v};
-        memcpy(&r, two, sizeof r);
-        return r;
-    };
-    Mult2 p;
-    for (int a = 0; a < 3; ++a) {
-        p.cA[a] = dup(m.cA[a]);
-        p.cD[a] = dup(m.cD[a]);
-        p.cE[a] = dup(m.cE[a]);
-        p.ncE[a] = dup(-m.cE[a]);
-        for (int b = 0; b < 3; ++b) p.cB[a][b] = dup(m.cB[a][b]);
-    }
-    return p;
-}
 
 constexpr int W = 4;                                            // cells per thread (along x)
 constexpr int TX = 64, TY = 8, D = 1;   // z-chunk length: launch parameter (zchunk_len)
@@ -535,12 +511,13 @@ static int tiles32(const Geom& g) {
 // idle work, but even where most of it is idle the kernel is the faster one (us a step, this kernel
 // and the two reference-form kernels: 300 x 250 x 112 109 / 225, 132 x 130 x 200 65 / 109,
 // 16 x 300 x 300 66 / 111, 32^3 8.6 / 10.7, 68 x 9 x 64 10.6 / 10.5).
-// Ragged grids of fewer than four planes stay with the reference form: the march forms two B
-// planes and reads five E planes for each chunk's first one (1000 x 750 x 1: 27 us against 24).
-bool fused32_supported(const Geom& g) {
+// Planes that do not couple along z (flat) take the 2D kernel (fdtd_step2d.cu); a coupled ragged
+// grid of fewer than four planes stays with the reference form, as the march forms two B planes
+// and reads five E planes for each chunk's first one.
+bool fused32_supported(const Geom& g, bool flat) {
     using namespace f32seg;
     const bool whole = g.nx % TX == 0 && g.ny % TY == 0;
-    return g.nx >= 2 * PX && g.ny >= 2 * PY && (whole || g.nz >= 4) &&
+    return g.nx >= 2 * PX && g.ny >= 2 * PY && (whole || flat || g.nz >= 4) &&
            g.total < (1LL << 31);   // 32-bit element offsets
 }
 

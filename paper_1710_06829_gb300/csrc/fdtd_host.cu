@@ -464,16 +464,17 @@ int fdtd_create(const fdtd_grid* grid, const double dx[3], double dt, const fdtd
     const char* env_split = getenv("FDTD_ADJOINT_SPLIT");
     h->adj_split = env_split && env_split[0] == '1';
     if (h->use_fused) {
+        const bool flat = G.nz == 1 || G.batched;
         if (G.dtype == FDTD_F32) {
             float* s0[6];
             float* s1[6];
             for (int c = 0; c < 6; ++c) { s0[c] = (float*)h->arr(0, c); s1[c] = (float*)h->arr(1, c); }
-            h->plan = fused_plan_create<float>(h->g, s0, s1);
+            h->plan = fused_plan_create<float>(h->g, flat, s0, s1);
         } else {
             double* s0[6];
             double* s1[6];
             for (int c = 0; c < 6; ++c) { s0[c] = (double*)h->arr(0, c); s1[c] = (double*)h->arr(1, c); }
-            h->plan = fused_plan_create<double>(h->g, s0, s1);
+            h->plan = fused_plan_create<double>(h->g, flat, s0, s1);
         }
     }
     *out = h;

@@ -115,10 +115,11 @@ void launch_ampere_v0(const Geom& g, const Mult<T>& m, FieldSet<T> s, const T* s
 // (E^{n+1}, B^{n+1/2}) to `out` (padded, images included).  hist_E (entries
 // nullable) receives E^{n+1}.  The plan holds the TMA descriptors of both sets.
 struct FusedPlan;
+// flat: the planes do not couple along z (nz = 1, or a batch of 2D problems)
 template <typename T>
-bool fused_supported(const Geom& g);
+bool fused_supported(const Geom& g, bool flat);
 template <typename T>
-FusedPlan* fused_plan_create(const Geom& g, T* const set0[6], T* const set1[6]);
+FusedPlan* fused_plan_create(const Geom& g, bool flat, T* const set0[6], T* const set1[6]);
 void fused_plan_destroy(FusedPlan* p);
 template <typename T>
 void launch_step_fused(const FusedPlan* plan, int in_set, const Geom& g, const Mult<T>& m,

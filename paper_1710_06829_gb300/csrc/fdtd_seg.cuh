@@ -4,6 +4,8 @@
 // their periodic images (the ghosts of the padded layout).
 #pragma once
 
+#include <cstring>
+
 #include "fdtd_tma.cuh"
 
 namespace fdtd {
@@ -197,6 +199,29 @@ __device__ __forceinline__ u64 fma2(u64 a, u64 b, u64 c) {
 }
 __device__ __forceinline__ u64 lo2(const Q4& q) { return pk(q.v[0], q.v[1]); }
 __device__ __forceinline__ u64 hi2(const Q4& q) { return pk(q.v[2], q.v[3]); }
+
+// the FP32 multipliers, each duplicated into a pair for the paired arithmetic
+struct Mult2 {
+    u64 cA[3], cD[3], cB[3][3], cE[3], ncE[3];   // ncE = -cE
+};
+
+inline Mult2 make_mult2(const Mult<float>& m) {
+    auto dup = [](float v) {
+        u64 r;
+        const float two[2] = {v, v};
+        memcpy(&r, two, sizeof r);
+        return r;
+    };
+    Mult2 p;
+    for (int a = 0; a < 3; ++a) {
+        p.cA[a] = dup(m.cA[a]);
+        p.cD[a] = dup(m.cD[a]);
+        p.cE[a] = dup(m.cE[a]);
+        p.ncE[a] = dup(-m.cE[a]);
+        for (int b = 0; b < 3; ++b) p.cB[a][b] = dup(m.cB[a][b]);
+    }
+    return p;
+}
 
 // dstar_diff on a pair of cells, with the transverse sums already formed:
 //   cA d_a + cD (f_a2 - f_am1) + cBb sb + cBc sc, in the order of dstar_diff

@@ -178,7 +178,7 @@ def _step_pair(shape, dtype, monkeypatch, steps=5, dims=3, **kw):
         sm = _sim(shape, dtype, dims, **kw)
         sm.set_state(f)
         src = None
-        if dims == 3 and not kw.get("batched"):
+        if not kw.get("batched"):
             src = S.Bunch(1.0, 0.9, 3.0, 2.0, 1.0, 2.0, 2.0)
         sm.step(steps, source=src)
         sm.sync()
@@ -221,3 +221,15 @@ def test_probe_loss_sums_the_plane(shape, dtype):
         ref += float(((sm.get_state()[2][:, :, nx - 1].double() - tgt[s].double()) ** 2).sum())
     assert abs(float(loss) - ref) <= 1e-12 * ref
     sm.close()
+
+
+# narrowest plane, whole tiles, last tiles of one column group or one row, tall and wide planes
+@pytest.mark.parametrize("nz,batched", [(1, False), (3, True), (1, None)])
+@pytest.mark.parametrize("nx,ny", [(8, 4), (64, 16), (68, 17), (60, 33), (1000, 5), (12, 300)])
+@pytest.mark.parametrize("dtype", ["f32", "f64"])
+def test_planes_step_bitwise_like_the_reference_form(nx, ny, nz, batched, dtype, monkeypatch):
+    """The 2D kernels on one plane (2D, and 3D one plane thick: batched None) and on a batch with its
+    layers on y; the one-plane runs carry the bunch current."""
+    kw = dict(batched=True, absorb_cells=2, absorb_sigma=0.3) if batched else {}
+    for a, b in zip(*_step_pair((nx, ny, nz), dtype, monkeypatch, dims=3 if batched is None else 2, **kw)):
+        assert torch.equal(a, b)
