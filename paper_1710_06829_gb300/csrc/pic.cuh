@@ -45,8 +45,13 @@ struct PushArgs {
     T escale[3];   // q / (dx_b dx_c): the cumulative shape change of axis a times this is -dt J_a
     int* err;
 };
+// mean: B0 holds B^n itself (launch_bmean) and B1 is not read.
 template <typename T>
-void launch_pic_push(const PushArgs<T>& a, cudaStream_t st);
+void launch_pic_push(const PushArgs<T>& a, bool mean, cudaStream_t st);
+
+// out = (b0 + b1) / 2 over n elements (n a multiple of 4)
+template <typename T>
+void launch_bmean(long long n, const T* b0, const T* b1, T* out, cudaStream_t st);
 
 // Copy every owned cell that has periodic images (the ghosts of the padded layout) to them,
 // for three padded arrays.

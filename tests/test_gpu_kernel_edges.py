@@ -233,3 +233,56 @@ def test_planes_step_bitwise_like_the_reference_form(nx, ny, nz, batched, dtype,
     kw = dict(batched=True, absorb_cells=2, absorb_sigma=0.3) if batched else {}
     for a, b in zip(*_step_pair((nx, ny, nz), dtype, monkeypatch, dims=3 if batched is None else 2, **kw)):
         assert torch.equal(a, b)
+
+
+# one warp, a ragged warp, several blocks; particles of one cell moving across no, one or three faces
+# and both ways along an axis (momenta along the cell's diagonal, or random), grids of a few cells, the
+# per-cell mean of B (at least 2^20 particles and one per cell)
+@pytest.mark.parametrize("sponge", [False, True])
+@pytest.mark.parametrize("shape,n,kind", [
+    ((8, 6, 5), 32, "diagonal"), ((8, 6, 5), 33, "random"), ((4, 4, 4), 700, "random"),
+    ((12, 8, 6), 64, "still"), ((8, 8, 8), 96, "along"), ((16, 12, 10), 5000, "random"),
+    ((32, 20, 16), 1 << 20, "random")])
+def test_push_and_current_match_the_oracle(shape, n, kind, sponge):
+    """Three cycles in FP64 against the oracle: every sum has at most n / cells + 60 terms a step, each
+    with a few eps; 1e-10 of the largest value covers 2^20 particles on 10^4 cells."""
+    from oracle import dispersion as D
+    from oracle import fdtd as F
+    from oracle import pic as P
+    from paper_1710_06829_gb300 import inputs
+    from paper_1710_06829_gb300 import sim as S
+    if n > 100000 and sponge:
+        pytest.skip("one large run is enough")
+    nx, ny, nz = shape
+    beta, delta = inputs.isotropic_theta(-0.05, -0.04, 0.02, 0.01)
+    dx = [1.0, 1.1, 0.9]
+    dt = 0.95 * D.dt_max(beta, delta, dx, 3)
+    rng = np.random.default_rng(n)
+    L = np.array([nx * dx[0], ny * dx[1], nz * dx[2]])[:, None]
+    if kind == "random":
+        x, u = rng.uniform(0, 1, (3, n)) * L, 2.0 * rng.standard_normal((3, n))
+    else:   # all in one cell
+        x = (rng.uniform(0, 1, (3, n)) + np.array([[nx - 1], [1], [0]])) * np.array(dx)[:, None]
+        d = {"diagonal": (4.0, 4.0, -4.0), "still": (0.0, 0.0, 0.0), "along": (9.0, 0.1, 0.0)}[kind]
+        u = np.repeat(np.array(d)[:, None], n, axis=1)
+    x[:, 0] = 0.0
+    f = [0.1 * a for a in inputs.random_fields(shape, 7)]
+    kw = dict(absorb_cells=2, absorb_sigma=0.3) if sponge else {}
+    sm = S.Simulation(shape, dx, dt, beta, delta, dtype="f64", **kw)
+    sm.set_state([torch.from_numpy(a) for a in f])
+    q = 1.0 / max(1, n // 100)
+    sp = S.Species(torch.from_numpy(x.copy()).cuda(), torch.from_numpy(u.copy()).cuda(), q, -1.0)
+    st, pt = F.State(f[:3], f[3:]), P.Particles(x, u, q, -1.0)
+    fac = F.sponge_factor((nz, ny, nx), 2, 0.3) if sponge else None
+    c = F.Coeffs(beta, delta, dx, dt)
+    for _ in range(3):
+        st = P.pic_step(st, [pt], c, fac)
+    sm.pic_step(3, [sp])
+    sm.sync()
+    got = [t.cpu().numpy() for t in sm.get_state()]
+    for a, b in zip(got, st.E + st.B):
+        assert np.max(np.abs(a - b)) <= 1e-10 * max(np.max(np.abs(v)) for v in st.E + st.B)
+    d = np.abs(sp.x.cpu().numpy() - pt.x)
+    assert np.max(np.minimum(d, L - d)) <= 1e-9   # a position on the seam may sit at either end
+    assert np.max(np.abs(sp.u.cpu().numpy() - pt.u)) <= 1e-9 * np.max(np.abs(pt.u)) + 1e-9
+    sm.close()
