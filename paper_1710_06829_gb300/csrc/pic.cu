@@ -35,8 +35,8 @@
 //   - where all 32 particles of a warp sit in one cell (a dense bunch, particles kept in cell
 //     order), the values of each face are summed through shared memory and added once.
 // Push per cycle: bunch of 2^22 particles in a 512 x 256 x 256 grid 717 -> 214 us; 2^22 particles of
-// a 128^3 plasma, drifted by a cell, 823 -> 332 us, bound by L2 (72 % busy: 10 sectors of additions
-// and 11 of loads a particle) and L1 (76 %).
+// a 128^3 plasma, drifted by a cell, 823 -> 317 us (332 with single additions instead of add_pair),
+// bound by L2 (72 % busy: 10 sectors of additions and 11 of loads a particle) and L1 (76 %).
 #include <climits>
 #include <cmath>
 
@@ -148,6 +148,27 @@ __device__ __forceinline__ void add_to(T* p, T v) {
     if (v != T(0)) atomicAdd(p, v);
 }
 
+// Adds v0, v1 at the x nodes f, f + 1 of a row (offset o of node f; f + 1 wraps only where o % 4 == 3):
+// one 16-byte reduction of the aligned group of four that holds both, which L2 takes as one
+// sector, where there is one.
+template <typename T, typename I>
+__device__ __forceinline__ void add_pair(T* row, I o, I o1, T v0, T v1) {
+    if constexpr (sizeof(T) == 4) {
+        const int r = (int)(o & 3);
+        if (r != 3) {
+            if (v0 == T(0) && v1 == T(0)) return;
+            const float a = r == 0 ? v0 : 0.0f, b = r == 0 ? v1 : r == 1 ? v0 : 0.0f,
+                        c = r == 1 ? v1 : r == 2 ? v0 : 0.0f, d = r == 2 ? v1 : 0.0f;
+            asm volatile("red.relaxed.gpu.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(row + (o - r)),
+                         "f"(a), "f"(b), "f"(c), "f"(d)
+                         : "memory");
+            return;
+        }
+    }
+    add_to(row + o, v0);
+    add_to(row + o1, v1);
+}
+
 // weight of the transverse nodes b, c of a face
 template <typename T, typename I>
 __device__ __forceinline__ T face_weight(const Move<T, I>& B, int b, const Move<T, I>& C, int c) {
@@ -179,8 +200,22 @@ __device__ __forceinline__ void deposit_lane(const PushArgs<T>& a, const Move<T,
         for (int q = 0; q < 4; ++q) f(q >> 1, q & 1);
     };
     if (cx != T(0)) all4([&](int b, int c) { jx(cx, X.o[0], b, c); });
-    if (cy != T(0)) all4([&](int b, int c) { jy(cy, Y.o[0], sy[0], b, c); });
-    if (cz != T(0)) all4([&](int b, int c) { jz(cz, Z.o[0], sz[0], b, c); });
+    if (cy != T(0)) {
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+            const T v = SP ? cy * (sy[0] * sz[c]) : cy;
+            add_pair(a.Eout[1] + (Y.o[0] + Z.o[c]), X.o[0], X.o[1], v * face_weight(X, 0, Z, c),
+                     v * face_weight(X, 1, Z, c));
+        }
+    }
+    if (cz != T(0)) {
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+            const T v = SP ? cz * (sy[c] * sz[0]) : cz;
+            add_pair(a.Eout[2] + (Y.o[c] + Z.o[0]), X.o[0], X.o[1], v * face_weight(X, 0, Y, c),
+                     v * face_weight(X, 1, Y, c));
+        }
+    }
     if (X.s) {
         all4([&](int b, int c) { jx(dx, X.ox, b, c); });
 #pragma unroll
