@@ -279,9 +279,14 @@ void launch_step2d32(const Geom& g, const Mult<float>& m, FieldSet<float> in, Fi
                      const float* spy, const float* spz, const float* jyz, const float* jx_row,
                      float* hist_E[3], int* err, cudaStream_t st);
 
+void launch_step2d64(const Geom& g, const Mult<double>& m, FieldSet<double> in, FieldSet<double> out,
+                     const double* spy, const double* spz, const double* jyz, const double* jx_row,
+                     double* hist_E[3], int* err, cudaStream_t st);
+
 template <typename T>
 bool fused_supported(const Geom& g, bool flat) {
     if constexpr (std::is_same<T, float>::value) return fused32_supported(g, flat);
+    if (flat) return true;   // fdtd_step2d64.cu takes every size
     using C = FusedCfg<T>;
     return g.nx % C::TX == 0 && g.ny % C::TY == 0 && g.nx >= C::TX && g.ny >= C::TY;
 }
@@ -318,6 +323,7 @@ FusedPlan* fused_plan_create(const Geom& g, bool flat, T* const set0[6], T* cons
     p->dtype = sizeof(T) == 4 ? FDTD_F32 : FDTD_F64;
     p->flat = flat;
     using Lc = Layout<T>;
+    if (std::is_same<T, double>::value && flat) return p;   // no descriptors
     for (int s = 0; s < 2; ++s) {
         T* const* set = s == 0 ? set0 : set1;
         for (int c = 0; c < 3; ++c) {
@@ -401,6 +407,11 @@ void launch_step_fused(const FusedPlan* plan, int in_set, const Geom& g, const M
                        err, st);
         return;
     }
+    if constexpr (std::is_same<T, double>::value)
+        if (plan->flat) {
+            launch_step2d64(g, m, in, out, sponge_y, sponge_z, jyz, jx_row, hist_E, err, st);
+            return;
+        }
     using C = FusedCfg<T>;
     const int nblk = (g.nx / C::TX) * (g.ny / C::TY) * ((g.nz + C::TZ - 1) / C::TZ);
     step_fused_kernel<T><<<nblk, C::NT, Layout<T>::SMEM, st>>>(

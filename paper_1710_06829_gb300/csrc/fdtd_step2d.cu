@@ -14,8 +14,8 @@
 // A thread works on segments of four cells as there (fdtd_seg.cuh).
 //
 // Bound: launch and latency for a small plane, HBM and L2 for a large batch.  Us a step, the 3D kernel (whole tiles) or
-// the reference form before and this kernel: 128 x 128 33 / 4.2, 1000 x 750 24 / 10.3, 512 x 512 x 32
-// 107 / 80 (805 MB: 0.74 of the copy rate).
+// the reference form before and this kernel: 128 x 128 33 / 2.8 (4.2 without the dependent launch),
+// 1000 x 750 24 / 7.9 (10.3), 512 x 512 x 32 107 / 77 (80; 805 MB: 0.77 of the copy rate).
 #include "fdtd_seg.cuh"
 
 namespace fdtd {
@@ -43,6 +43,8 @@ step2d_kernel(Geom g, Mult<float> m, Mult2 m2, FieldSet<float> in, FieldSet<floa
               int* __restrict__ err) {
     __shared__ __align__(16) float sE[3 * EPL];
     __shared__ __align__(16) float sB[3 * BPL];
+    pdl_trigger();
+    pdl_wait();
     const int ntx = (g.nx + TX - 1) / TX, nty = (g.ny + TY - 1) / TY;
     int w = blockIdx.x;
     const int tx = w % ntx;
@@ -176,8 +178,8 @@ void launch_step2d32(const Geom& g, const Mult<float>& m, FieldSet<float> in, Fi
                      float* hist_E[3], int* err, cudaStream_t st) {
     using namespace flat32;
     const long long tiles = (long long)((g.nx + TX - 1) / TX) * ((g.ny + TY - 1) / TY) * g.nz;
-    step2d_kernel<<<(unsigned)tiles, NT, 0, st>>>(g, m, make_mult2(m), in, out, spy, spz, jyz, jx_row,
-                                                  hist_E[0], hist_E[1], hist_E[2], err);
+    launch_pdl(step2d_kernel, dim3((unsigned)tiles), dim3(NT), 0, st, g, m, make_mult2(m), in, out, spy,
+               spz, jyz, jx_row, hist_E[0], hist_E[1], hist_E[2], err);
 }
 
 }  // namespace fdtd

@@ -19,6 +19,33 @@ struct FusedPlan {
     FusedMaps maps[2];   // indexed by input set
 };
 
+// ---------------------------------------------------------------- dependent launches
+
+// Launch `k` so that it may be set up while the kernel before it in the stream still runs
+// (programmatic dependent launch): its blocks start when every block of that kernel has called
+// pdl_trigger() or ended, and pdl_wait() returns when that kernel has completed and its writes are
+// visible.  A kernel launched this way calls pdl_wait() in every thread before it touches global
+// memory.  Between the steps of a time loop this hides about 2 us of launch latency.
+template <class... P, class... A>
+inline void launch_pdl(void (*k)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... a) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, k, P(a)...);   // the caller looks at cudaGetLastError()
+}
+
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 // ---------------------------------------------------------------- PTX helpers
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
