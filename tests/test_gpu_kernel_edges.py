@@ -193,12 +193,19 @@ RAGGED = [(8, 4, 4), (60, 12, 5), (64, 9, 4), (68, 8, 7), (132, 31, 4), (124, 30
 
 
 @pytest.mark.parametrize("sponge", [False, True])
+@pytest.mark.parametrize("dtype", ["f32", "f64"])
 @pytest.mark.parametrize("shape", RAGGED)
-def test_ragged_tiles_step_bitwise_like_the_reference_form(shape, sponge, monkeypatch):
+def test_ragged_tiles_step_bitwise_like_the_reference_form(shape, dtype, sponge, monkeypatch):
     if sponge and min(shape[1:]) < 4:
         pytest.skip("no room for the layers")
     kw = dict(absorb_cells=2, absorb_sigma=0.3) if sponge else {}
-    for a, b in zip(*_step_pair(shape, "f32", monkeypatch, **kw)):
+    for a, b in zip(*_step_pair(shape, dtype, monkeypatch, **kw)):
+        assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("shape", [(4, 2, 2), (4, 16, 3), (32, 3, 9), (64, 48, 33)])
+def test_fp64_step_on_grids_inside_one_tile_and_whole_tiles(shape, monkeypatch):
+    for a, b in zip(*_step_pair(shape, "f64", monkeypatch)):
         assert torch.equal(a, b)
 
 
