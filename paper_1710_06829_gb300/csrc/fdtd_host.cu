@@ -69,6 +69,9 @@ void launch_adjoint32_fused(const FusedMaps& maps, const Geom& g, const Mult<flo
 void launch_adjoint32_E(const FusedMaps& maps, const Geom& g, const Mult<float>& m,
                         FieldSet<float> lam, const float* spy, const float* spz, int* err,
                         cudaStream_t st);
+int adjoint64_blocks(const Geom& g);
+void launch_adjoint64(const Geom& g, const Mult<double>& m, FieldSet<double> lam, const double* const E[3],
+                      const double* spy, const double* spz, double* partials, cudaStream_t st);
 template <typename T>
 void launch_energy(const Geom& g, FieldSet<T> s, int x_lo, int x_len, int my, int mz, double dV,
                    double* part, double* out, cudaStream_t st);
@@ -986,7 +989,9 @@ static int adjoint_impl(fdtd_handle* h, int n, const fdtd_probe* probe, double* 
     if (rc) return rc;
     const bool staged = std::is_same<T, float>::value && !h->hist_maps.empty();
     const bool one_kernel = std::is_same<T, float>::value && h->lam_fused;
-    const int nblk = one_kernel ? adjoint32f_blocks(g) : staged ? adjoint32_blocks(g) : adjoint_B_blocks(g);
+    const bool tiled64 = std::is_same<T, double>::value && h->plan != nullptr;
+    const int nblk = one_kernel ? adjoint32f_blocks(g) : staged ? adjoint32_blocks(g)
+                     : tiled64 ? adjoint64_blocks(g) : adjoint_B_blocks(g);
     if (h->npart < nblk) {
         if (h->partials) cudaFree(h->partials);
         h->partials = nullptr;
@@ -1016,6 +1021,13 @@ static int adjoint_impl(fdtd_handle* h, int n, const fdtd_probe* probe, double* 
                                        h->partials, h->err_dev, h->stream);
                 CK(cudaGetLastError());
                 h->lam_cur ^= 1;
+                continue;
+            }
+        }
+        if constexpr (std::is_same<T, double>::value) {
+            if (tiled64) {
+                launch_adjoint64(g, m, lam, E, spy, spz, h->partials, h->stream);
+                CK(cudaGetLastError());
                 continue;
             }
         }

@@ -293,3 +293,35 @@ def test_push_and_current_match_the_oracle(shape, n, kind, sponge):
     assert np.max(np.minimum(d, L - d)) <= 1e-9   # a position on the seam may sit at either end
     assert np.max(np.abs(sp.u.cpu().numpy() - pt.u)) <= 1e-9 * np.max(np.abs(pt.u)) + 1e-9
     sm.close()
+
+
+@pytest.mark.parametrize("sponge", [False, True])
+@pytest.mark.parametrize("shape", RAGGED + [(4, 2, 2), (4, 3, 5), (32, 3, 9), (64, 48, 33)])
+def test_fp64_reverse_step_matches_the_reference_form(shape, sponge, monkeypatch):
+    """lambda and the coefficient gradient of three recorded steps, with a probe on the last column.
+    Per value about 40 FP64 operations a reverse step on terms of the field's size: 3 x 40 x 2^-53 =
+    1.3e-14 of the largest value; 1e-13 taken, and for the gradient's sums of up to 4e5 terms 1e-11
+    of the largest entry."""
+    if sponge and min(shape[1:]) < 4:
+        pytest.skip("no room for the layers")
+    from paper_1710_06829_gb300 import sim as S
+    kw = dict(absorb_cells=2, absorb_sigma=0.3) if sponge else {}
+    f = [torch.from_numpy(a) for a in _random_state(shape, "f64", 12)]
+    lam = [torch.from_numpy(a) for a in _random_state(shape, "f64", 13)]
+    nx, ny, nz = shape
+    tgt = torch.from_numpy(np.random.default_rng(3).standard_normal((3, nz, ny))).cuda()
+    out = []
+    for flag in ("1", "0"):
+        monkeypatch.setenv("FDTD_FUSED", flag)
+        sm = _sim(shape, "f64", **kw)
+        sm.set_state(f)
+        sm.step(3, record=True)
+        sm.set_adjoint(lam)
+        grad = torch.zeros(12, dtype=torch.float64, device="cuda")
+        sm.step_adjoint(3, grad, probe=S.Probe(1, nx - 1, tgt))
+        out.append((sm.get_adjoint(), grad.cpu()))
+        sm.sync()
+        sm.close()
+    for a, b in zip(out[0][0], out[1][0]):
+        assert float((a - b).abs().max()) <= 1e-13 * max(float(c.abs().max()) for c in out[1][0])
+    assert float((out[0][1] - out[1][1]).abs().max()) <= 1e-11 * float(out[1][1].abs().max())
