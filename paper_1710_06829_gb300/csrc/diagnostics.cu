@@ -14,7 +14,7 @@
 // Partials: one FP64 value (or pair) per block, summed in a fixed order by the last block.
 #include <cmath>
 
-#include "fdtd_internal.cuh"
+#include "fdtd_tma.cuh"
 
 namespace fdtd {
 
@@ -106,6 +106,8 @@ template <typename T>
 __global__ void __launch_bounds__(DG_THREADS)
 probe_loss_kernel(Geom g, const T* __restrict__ F, int xp, const T* __restrict__ target,
                   double* part, unsigned* ticket, double* loss) {
+    pdl_trigger();
+    pdl_wait();
     double acc[1] = {0.0};
     const long long n = (long long)g.ny * g.nz;
     for (long long t = (long long)blockIdx.x * DG_THREADS + threadIdx.x; t < n;
@@ -195,6 +197,8 @@ __device__ __forceinline__ Item item_at(const Geom& g, long long t) {
 // 67 MB that are read.
 __global__ void phase_kernel(Geom g, double kx, double ky, double kz, double ox, double oy,
                              double oz, double2* __restrict__ tab) {
+    pdl_trigger();
+    pdl_wait();
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t < g.nx) phase_entry(tab, t, kx, ox);
     else if (t < g.nx + g.ny) phase_entry(tab + g.nx, t - g.nx, ky, oy);
@@ -206,6 +210,8 @@ __global__ void __launch_bounds__(DG_THREADS)
 planewave_kernel(Geom g, const T* __restrict__ F, const double2* __restrict__ tab, double* part,
                  unsigned* ticket, double* out) {
     constexpr int V = Vec<T>::N;
+    pdl_trigger();
+    pdl_wait();
     double acc[2] = {0.0, 0.0};
     const long long n = item_count<T>(g);
     for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < n;
@@ -430,8 +436,8 @@ template <typename T>
 void launch_probe_loss(const Geom& g, const T* E, int x_index, const T* target, double* scratch,
                        double* loss, cudaStream_t st) {
     const DiagScratch d = diag_scratch(g, scratch);
-    probe_loss_kernel<T><<<blocks_of((long long)g.ny * g.nz, g), DG_THREADS, 0, st>>>(
-        g, E, x_index, target, d.part, d.ticket, loss);
+    launch_pdl(probe_loss_kernel<T>, dim3(blocks_of((long long)g.ny * g.nz, g)), dim3(DG_THREADS), 0, st, g,
+               E, x_index, target, d.part, d.ticket, loss);
 }
 template void launch_probe_loss<float>(const Geom&, const float*, int, const float*, double*,
                                        double*, cudaStream_t);
@@ -443,9 +449,10 @@ void launch_planewave(const Geom& g, const T* F, const double k[3], const double
                       double* scratch, double* out, cudaStream_t st) {
     const DiagScratch d = diag_scratch(g, scratch);
     const int lines = g.nx + g.ny + g.nz;
-    phase_kernel<<<(lines + 63) / 64, 64, 0, st>>>(g, k[0], k[1], k[2], off[0], off[1], off[2], d.tab);
-    planewave_kernel<T><<<blocks_of(item_count<T>(g), g), DG_THREADS, 0, st>>>(g, F, d.tab, d.part,
-                                                                               d.ticket, out);
+    launch_pdl(phase_kernel, dim3((lines + 63) / 64), dim3(64), 0, st, g, k[0], k[1], k[2], off[0], off[1],
+               off[2], d.tab);
+    launch_pdl(planewave_kernel<T>, dim3(blocks_of(item_count<T>(g), g)), dim3(DG_THREADS), 0, st, g, F, d.tab,
+               d.part, d.ticket, out);
 }
 
 template <typename T>

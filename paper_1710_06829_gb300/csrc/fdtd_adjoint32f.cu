@@ -298,6 +298,8 @@ adjF_kernel(const __grid_constant__ FusedMaps maps, Geom g, Mult<float> m, Field
     __syncthreads();
     tm_fence_after();
     const uint32_t tb = *tm_slot + ((uint32_t)(32 * (wq & 3)) << 16);
+    pdl_trigger();   // nothing above touches global memory
+    pdl_wait();
     auto cmu = [&](int c, int sl) { return tb + (uint32_t)(4 * (c * NM + sl)); };
     auto cle = [&](int c, int s3) { return tb + (uint32_t)(COL_LE + 4 * (3 * c + s3)); };
     int issued = 0;
@@ -646,9 +648,8 @@ void launch_adjoint32_fused(const FusedMaps& maps, const Geom& g, const Mult<flo
                             const float* spy, const float* spz, double* partials, int* err,
                             cudaStream_t st) {
     auto kern = spy != nullptr ? adj32f::adjF_kernel<true> : adj32f::adjF_kernel<false>;
-    kern<<<adjoint32f_blocks(g), adj32f::NT, adj32f::SMEM, st>>>(maps, g, m, lam, out, E[0], E[1],
-                                                                  E[2], spy, spz, partials,
-                                                                  adjoint32f_tz(g), err);
+    launch_pdl(kern, dim3((unsigned)adjoint32f_blocks(g)), dim3(adj32f::NT), adj32f::SMEM, st, maps, g, m,
+               lam, out, E[0], E[1], E[2], spy, spz, partials, adjoint32f_tz(g), err);
 }
 
 }  // namespace fdtd

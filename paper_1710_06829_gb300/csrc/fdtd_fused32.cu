@@ -175,6 +175,10 @@ step_kernel(const __grid_constant__ FusedMaps maps, Geom g, Mult<float> m, Mult2
     tm_fence_after();
     const uint32_t tm_base = *tm_slot;
     const int warp = tid >> 5;
+    // the next kernel's blocks may be set up from here on (they take the slots that this one's last
+    // wave leaves); nothing above touches global memory
+    pdl_trigger();
+    pdl_wait();
     // this thread's TMEM lane (quadrant of its warp) and column base
     const uint32_t tb = tm_base + ((uint32_t)(32 * (warp & 3)) << 16) + (warp == 4 ? COL_HALO : 0);
     int issued = 0;
@@ -624,8 +628,8 @@ void launch_fused32(const FusedMaps& maps, FieldSet<float> in, const Geom& g, co
     using namespace f32seg;
     const int tz = fused32_tz(g);
     const int nblk = tiles32(g) * ((g.nz + tz - 1) / tz);
-    step_kernel<<<nblk, NT, SMEM, st>>>(maps, g, m, make_mult2(m), in, out, spy, spz, jyz, jx_row, hist_E[0],
-                                        hist_E[1], hist_E[2], 0, g.nz, tz, err);
+    launch_pdl(step_kernel, dim3((unsigned)nblk), dim3(NT), SMEM, st, maps, g, m, make_mult2(m), in, out, spy,
+               spz, jyz, jx_row, hist_E[0], hist_E[1], hist_E[2], 0, g.nz, tz, err);
 }
 
 // One leapfrog step on the planes zs .. ze-1 only (no current, no history): the slab launches
@@ -641,8 +645,8 @@ void launch_fused32_range(const FusedMaps& maps, FieldSet<float> in, const Geom&
     const int len = ze - zs;
     const int tz = zchunk_len(tiles, len, slots, 2, 64);
     const int nblk = tiles * ((len + tz - 1) / tz);
-    step_kernel<<<nblk, NT, SMEM, st>>>(maps, g, m, make_mult2(m), in, out, spy, spz, nullptr,
-                                        nullptr, nullptr, nullptr, nullptr, zs, ze, tz, err);
+    launch_pdl(step_kernel, dim3((unsigned)nblk), dim3(NT), SMEM, st, maps, g, m, make_mult2(m), in, out, spy,
+               spz, nullptr, nullptr, nullptr, nullptr, nullptr, zs, ze, tz, err);
 }
 
 }  // namespace fdtd

@@ -13,7 +13,7 @@
 //   E_x += dt (D_y B_z - D_z B_y - J_x), and cyclically.
 #include <cmath>
 
-#include "fdtd_internal.cuh"
+#include "fdtd_tma.cuh"
 #include "pic.cuh"
 
 namespace fdtd {
@@ -508,6 +508,8 @@ template void launch_pack<double>(const Geom&, const double* const[6], double* c
 template <typename T>
 __global__ void probe_adjoint_kernel(Geom g, T* __restrict__ lam, const T* __restrict__ F, int xp,
                                      const T* __restrict__ target) {
+    pdl_trigger();
+    pdl_wait();
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= g.ny * g.nz) return;
     const int j = t % g.ny, k = t / g.ny;
@@ -520,7 +522,7 @@ template <typename T>
 void launch_probe_adjoint(const Geom& g, T* lamE, const T* E, int x_index, const T* target,
                           cudaStream_t st) {
     const int n = g.ny * g.nz;
-    probe_adjoint_kernel<T><<<(n + 255) / 256, 256, 0, st>>>(g, lamE, E, x_index, target);
+    launch_pdl(probe_adjoint_kernel<T>, dim3((n + 255) / 256), dim3(256), 0, st, g, lamE, E, x_index, target);
 }
 template void launch_probe_adjoint<float>(const Geom&, float*, const float*, int, const float*,
                                           cudaStream_t);
