@@ -65,103 +65,106 @@ __device__ __forceinline__ void dcoef(const T* __restrict__ F, long long c, long
     dc = (F[c + a1 + cp] - F[c + cp]) + (F[c + a1 + cm] - F[c + cm]) - T(2) * ax;
 }
 
-constexpr int ADJ_THREADS = 256;
+// The cells are summed in chains: chain (b, t) holds the cells i = t, t + 256, ... of the rows b,
+// b + CHAIN_ROWS, ... in that order, at most ADJ_FLUSH of their terms in the field precision before
+// they are added to FP64 accumulators (an FP64 add costs 64 issue slots on this part).  The chains
+// fix the rounding of an FP32 gradient, so they stay as they are; which thread takes a chain does
+// not matter, so the threads take them one after the other, the chains of a row on neighbouring
+// threads (one block a chain row left most lanes of a narrow grid idle and, at 140 registers,
+// one block an SM: 418 us at 300 x 250 x 56 FP32, 180 here), and a block's sums are taken once.
+// Groups are a loop of their own: as a test in the cell loop the adds were made in every cell.
+constexpr int ADJ_THREADS = 128, CHAIN_WIDTH = 256, CHAIN_ROWS = 152 * 8, ADJ_FLUSH = 16;
+
+static long long adjoint_chains(const Geom& g) {
+    const long long rows = (long long)g.ny * g.nz;
+    return (rows < CHAIN_ROWS ? rows : CHAIN_ROWS) * (g.nx < CHAIN_WIDTH ? g.nx : CHAIN_WIDTH);
+}
 
 int adjoint_B_blocks(const Geom& g) {
-    long long b = (long long)g.ny * g.nz;   // one x-row per block and sweep
-    if (b > 152 * 8) b = 152 * 8;
-    return (int)b;
+    const long long b = (adjoint_chains(g) + ADJ_THREADS - 1) / ADJ_THREADS;
+    return (int)(b < 152 * 4 ? b : 152 * 4);   // the resident blocks
 }
 
 // partials layout: [block][9] = per axis a (x, y, z): d/d delta_a, d/d beta_a,b1, d/d beta_a,b2
 // with b1 < b2 the two other axes.  Accumulated across steps (+=) by the owning block.
-// A block walks whole x-rows (j, k); each thread sums at most ADJ_FLUSH cell terms in the
-// field precision before adding them to its FP64 accumulators, so the FP64 pipe (slow on
-// this part) sees one add per ADJ_FLUSH cells; block and grid totals are FP64.
-constexpr int ADJ_FLUSH = 16;
-
 template <typename T>
-__global__ void __launch_bounds__(ADJ_THREADS)
+__global__ void __launch_bounds__(ADJ_THREADS, sizeof(T) == 4 ? 4 : 2)
 adjoint_B_kernel(Geom g, Mult<T> m, FieldSet<T> lam, const T* __restrict__ Ex,
                  const T* __restrict__ Ey, const T* __restrict__ Ez, const T* __restrict__ spy,
                  const T* __restrict__ spz, double* __restrict__ partials) {
     double acc[9];
-    T racc[9];
 #pragma unroll
-    for (int q = 0; q < 9; ++q) {
-        acc[q] = 0.0;
-        racc[q] = T(0);
-    }
-    int cnt = 0;
+    for (int q = 0; q < 9; ++q) acc[q] = 0.0;
     const int rows = g.ny * g.nz;
+    const int nrow = rows < CHAIN_ROWS ? rows : CHAIN_ROWS, width = g.nx < CHAIN_WIDTH ? g.nx : CHAIN_WIDTH;
     const long long Y = g.nxp;
     const T* lEx = lam.c[0];
     const T* lEy = lam.c[1];
     const T* lEz = lam.c[2];
-    for (int r = blockIdx.x; r < rows; r += gridDim.x) {
-        const int j = r % g.ny, k = r / g.ny;
-        const long long rowbase = pidx(g, 0, j, k);
-        const long long zp1 = zoff_a(g, k, 1), zm1 = zoff_a(g, k, -1), zp2 = zoff_a(g, k, 2);
-        // l_E = S lambda_E at the cell and its +x, +y, +z neighbours
-        const T s0 = sp_at(g, spy, spz, j, k);
-        const T sxp = s0;
-        const T syp = sp_at(g, spy, spz, j + 1, k);
-        const T szp = sp_at(g, spy, spz, j, k + 1);
-        for (int i = threadIdx.x; i < g.nx; i += blockDim.x) {
-            const long long c = rowbase + i;
-            const T ex0 = s0 * lEx[c], ey0 = s0 * lEy[c], ez0 = s0 * lEz[c];
-            // G^T l_E (transposed backward differences = forward differences with a minus sign)
-            T nx_ = lam.c[3][c] + (m.cE[2] * (ey0 - szp * lEy[c + zp1]) - m.cE[1] * (ez0 - syp * lEz[c + Y]));
-            T ny_ = lam.c[4][c] + (m.cE[0] * (ez0 - sxp * lEz[c + 1]) - m.cE[2] * (ex0 - szp * lEx[c + zp1]));
-            T nz_ = lam.c[5][c] + (m.cE[1] * (ex0 - syp * lEx[c + Y]) - m.cE[0] * (ey0 - sxp * lEy[c + 1]));
-            const T mux = s0 * nx_, muy = s0 * ny_, muz = s0 * nz_;
-            // gradient: axis x appears as +mu_y D*_x E_z - mu_z D*_x E_y
-            T d0, d1, d2, e0, e1, e2;
-            dcoef(Ez, c, 1, 2, -1, Y, -Y, zp1, zm1, d0, d1, d2);
-            dcoef(Ey, c, 1, 2, -1, Y, -Y, zp1, zm1, e0, e1, e2);
-            racc[0] += muy * d0 - muz * e0;
-            racc[1] += muy * d1 - muz * e1;
-            racc[2] += muy * d2 - muz * e2;
-            // axis y: +mu_z D*_y E_x - mu_x D*_y E_z   (transverse order x, z)
-            dcoef(Ex, c, Y, 2 * Y, -Y, 1, -1, zp1, zm1, d0, d1, d2);
-            dcoef(Ez, c, Y, 2 * Y, -Y, 1, -1, zp1, zm1, e0, e1, e2);
-            racc[3] += muz * d0 - mux * e0;
-            racc[4] += muz * d1 - mux * e1;
-            racc[5] += muz * d2 - mux * e2;
-            // axis z: +mu_x D*_z E_y - mu_y D*_z E_x   (transverse order x, y)
-            dcoef(Ey, c, zp1, zp2, zm1, 1, -1, Y, -Y, d0, d1, d2);
-            dcoef(Ex, c, zp1, zp2, zm1, 1, -1, Y, -Y, e0, e1, e2);
-            racc[6] += mux * d0 - muy * e0;
-            racc[7] += mux * d1 - muy * e1;
-            racc[8] += mux * d2 - muy * e2;
-            if (++cnt == ADJ_FLUSH) {
+    for (int ch = blockIdx.x * ADJ_THREADS + threadIdx.x; ch < nrow * width; ch += gridDim.x * ADJ_THREADS) {
+        const int b = ch / width, t = ch - b * width;
+        for (int r = b, i = t; r < rows;) {
+            T racc[9];
 #pragma unroll
-                for (int q = 0; q < 9; ++q) {
-                    acc[q] += (double)racc[q];
-                    racc[q] = T(0);
+            for (int q = 0; q < 9; ++q) racc[q] = T(0);
+#pragma unroll 1
+            for (int cnt = 0; cnt < ADJ_FLUSH && r < rows; ++cnt) {
+                const int k = r / g.ny, j = r - k * g.ny;
+                const long long rowbase = pidx(g, 0, j, k);
+                const long long zp1 = zoff_a(g, k, 1), zm1 = zoff_a(g, k, -1), zp2 = zoff_a(g, k, 2);
+                // l_E = S lambda_E at the cell and its +x, +y, +z neighbours
+                const T s0 = sp_at(g, spy, spz, j, k);
+                const T sxp = s0;
+                const T syp = sp_at(g, spy, spz, j + 1, k);
+                const T szp = sp_at(g, spy, spz, j, k + 1);
+                const long long c = rowbase + i;
+                const T ex0 = s0 * lEx[c], ey0 = s0 * lEy[c], ez0 = s0 * lEz[c];
+                // G^T l_E (transposed backward differences = forward differences with a minus sign)
+                T nx_ = lam.c[3][c] + (m.cE[2] * (ey0 - szp * lEy[c + zp1]) - m.cE[1] * (ez0 - syp * lEz[c + Y]));
+                T ny_ = lam.c[4][c] + (m.cE[0] * (ez0 - sxp * lEz[c + 1]) - m.cE[2] * (ex0 - szp * lEx[c + zp1]));
+                T nz_ = lam.c[5][c] + (m.cE[1] * (ex0 - syp * lEx[c + Y]) - m.cE[0] * (ey0 - sxp * lEy[c + 1]));
+                const T mux = s0 * nx_, muy = s0 * ny_, muz = s0 * nz_;
+                // gradient: axis x appears as +mu_y D*_x E_z - mu_z D*_x E_y
+                T d0, d1, d2, e0, e1, e2;
+                dcoef(Ez, c, 1, 2, -1, Y, -Y, zp1, zm1, d0, d1, d2);
+                dcoef(Ey, c, 1, 2, -1, Y, -Y, zp1, zm1, e0, e1, e2);
+                racc[0] += muy * d0 - muz * e0;
+                racc[1] += muy * d1 - muz * e1;
+                racc[2] += muy * d2 - muz * e2;
+                // axis y: +mu_z D*_y E_x - mu_x D*_y E_z   (transverse order x, z)
+                dcoef(Ex, c, Y, 2 * Y, -Y, 1, -1, zp1, zm1, d0, d1, d2);
+                dcoef(Ez, c, Y, 2 * Y, -Y, 1, -1, zp1, zm1, e0, e1, e2);
+                racc[3] += muz * d0 - mux * e0;
+                racc[4] += muz * d1 - mux * e1;
+                racc[5] += muz * d2 - mux * e2;
+                // axis z: +mu_x D*_z E_y - mu_y D*_z E_x   (transverse order x, y)
+                dcoef(Ey, c, zp1, zp2, zm1, 1, -1, Y, -Y, d0, d1, d2);
+                dcoef(Ex, c, zp1, zp2, zm1, 1, -1, Y, -Y, e0, e1, e2);
+                racc[6] += mux * d0 - muy * e0;
+                racc[7] += mux * d1 - muy * e1;
+                racc[8] += mux * d2 - muy * e2;
+                store_images_a(g, lam.c[3], i, j, k, mux);
+                store_images_a(g, lam.c[4], i, j, k, muy);
+                store_images_a(g, lam.c[5], i, j, k, muz);
+                i += CHAIN_WIDTH;
+                if (i >= g.nx) {
+                    i = t;
+                    r += nrow;
                 }
-                cnt = 0;
             }
-            store_images_a(g, lam.c[3], i, j, k, mux);
-            store_images_a(g, lam.c[4], i, j, k, muy);
-            store_images_a(g, lam.c[5], i, j, k, muz);
+#pragma unroll
+            for (int q = 0; q < 9; ++q) acc[q] += (double)racc[q];
         }
     }
+    __shared__ double sm[9][ADJ_THREADS];
 #pragma unroll
-    for (int q = 0; q < 9; ++q) acc[q] += (double)racc[q];
-    __shared__ double red[ADJ_THREADS / 32][9];
-    const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-#pragma unroll
-    for (int q = 0; q < 9; ++q) {
-        double v = acc[q];
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-        if (l == 0) red[w][q] = v;
-    }
+    for (int q = 0; q < 9; ++q) sm[q][threadIdx.x] = acc[q];
     __syncthreads();
-    if (threadIdx.x < 9) {
-        double v = 0.0;
-        for (int ww = 0; ww < ADJ_THREADS / 32; ++ww) v += red[ww][threadIdx.x];
-        partials[(long long)blockIdx.x * 9 + threadIdx.x] += v;
+    const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+    for (int q = w; q < 9; q += ADJ_THREADS / 32) {
+        double v = (sm[q][l] + sm[q][l + 32]) + (sm[q][l + 64] + sm[q][l + 96]);
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+        if (l == 0) partials[(long long)blockIdx.x * 9 + q] += v;
     }
 }
 
