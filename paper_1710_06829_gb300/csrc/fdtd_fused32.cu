@@ -242,9 +242,20 @@ step_kernel(const __grid_constant__ FusedMaps maps, Geom g, Mult<float> m, Mult2
     float fin = 0.0f;   // non-finite detection (nonfinite_acc): stays 0 while every E value is finite
     int it = 0;
     {
-        bool ok0 = true;
-        if (tid == PRODUCER) ok0 = mbar_wait(&bar[NS], 0) && mbar_wait(&bar[0], 0);
+        const bool ok0 = mbar_wait(&bar[NS], 0) && mbar_wait(&bar[0], 0);
         failed = __syncthreads_or(!ok0);
+    }
+    if (!failed) {   // own rows of E planes z0-2 .. z0 (E_z: z0-2, z0-1) to their TMEM slots
+        const float *Pm = sE, *P0 = sE + 3 * ESLOT, *P1 = sE + 6 * ESLOT;
+        tm_st(tb + COL_EX, ldq(Pm, e));
+        tm_st(tb + COL_EX + 4, ldq(P0, e));
+        tm_st(tb + COL_EX + 8, ldq(P1, e));
+        tm_st(tb + COL_EY, ldq(Pm + ESLOT, e));
+        tm_st(tb + COL_EY + 4, ldq(P0 + ESLOT, e));
+        tm_st(tb + COL_EY + 8, ldq(P1 + ESLOT, e));
+        tm_st(tb + COL_EZ, ldq(Pm + 2 * ESLOT, e));
+        tm_st(tb + COL_EZ + 4, ldq(P0 + 2 * ESLOT, e));
+        tm_wait_st();
     }
     // plane bookkeeping by counters (no integer division in the loop):
     //   pw = p mod nz, qw = (p-1) mod nz, s_m = ring slot of plane p-1 = it mod NE,
@@ -266,10 +277,7 @@ step_kernel(const __grid_constant__ FusedMaps maps, Geom g, Mult<float> m, Mult2
         const float* P1 = sE + s_1 * 3 * ESLOT;
         const float* P2 = sE + s_2 * 3 * ESLOT;
         bool ok = true;
-        if (it < niter) {
-            if (it == 0) ok = mbar_wait(&bar[NS], 0);
-            ok = ok && mbar_wait(&bar[it % NS], (uint32_t)((it / NS) & 1));
-        }
+        if (it < niter) ok = mbar_wait(&bar[it % NS], (uint32_t)((it / NS) & 1));
         ok = __all_sync(FULL, ok);   // keeps the shuffles below warp-uniform
         // TMEM columns of the own rows: E_x, E_y of plane p-1+k in slot (it+k) & 3, E_z of plane
         // p-1+k in slot (it+k) mod 3; own B^{n+1/2} rows of plane p in slot it mod 3 (B_z: it & 1)
@@ -304,33 +312,16 @@ step_kernel(const __grid_constant__ FusedMaps maps, Geom g, Mult<float> m, Mult2
             u64 dz2[2], dy2[2], b2[3][2];
             float t[W];
             // own rows: the newest plane comes from shared memory (E_x, E_y of p+2; E_z of p+1)
-            // and goes to TMEM; the older planes come from TMEM (at the first iteration every
-            // own row comes from shared memory and is written to TMEM)
+            // and goes to TMEM; the older planes come from TMEM
             Q4 ym_, y0_, y1_, zm_, z0_, z1_;
             const Q4 y2_ = ldq(P2 + ESLOT, e);
             z1_ = ldq(P1 + 2 * ESLOT, e);
-            if (it == 0) {
-                ym_ = ldq(Pm + ESLOT, e);
-                y0_ = ldq(P0 + ESLOT, e);
-                y1_ = ldq(P1 + ESLOT, e);
-                zm_ = ldq(Pm + 2 * ESLOT, e);
-                z0_ = ldq(P0 + 2 * ESLOT, e);
-                tm_st(cx(0), ldq(Pm, e));
-                tm_st(cx(1), ldq(P0, e));
-                tm_st(cx(2), ldq(P1, e));   // read back from TMEM from the next iteration on
-                tm_st(cy(0), ym_);
-                tm_st(cy(1), y0_);
-                tm_st(cy(2), y1_);
-                tm_st(cz0, zm_);
-                tm_st(cz1, z0_);
-            } else {
-                tm_ld(cy(0), ym_);
-                tm_ld(cy(1), y0_);
-                tm_ld(cy(2), y1_);
-                tm_ld(cz0, zm_);
-                tm_ld(cz1, z0_);
-                tm_wait_ld(ym_, y0_, y1_, zm_, z0_);
-            }
+            tm_ld(cy(0), ym_);
+            tm_ld(cy(1), y0_);
+            tm_ld(cy(2), y1_);
+            tm_ld(cz0, zm_);
+            tm_ld(cz1, z0_);
+            tm_wait_ld(ym_, y0_, y1_, zm_, z0_);
             tm_st(cy(3), y2_);
             tm_st(cz2, z1_);
             // B_x = B_x + (D*_z E_y - D*_y E_z)
@@ -346,16 +337,10 @@ step_kernel(const __grid_constant__ FusedMaps maps, Geom g, Mult<float> m, Mult2
                      m.cA[0], m.cD[0], m.cB[0][1], m.cB[0][2], t);
             Q4 xm_, x0_, x1_;
             const Q4 x2_ = ldq(P2, e);
-            if (it == 0) {   // written to TMEM in this iteration: not read back before a wait
-                xm_ = ldq(Pm, e);
-                x0_ = ldq(P0, e);
-                x1_ = ldq(P1, e);
-            } else {
-                tm_ld(cx(0), xm_);
-                tm_ld(cx(1), x0_);
-                tm_ld(cx(2), x1_);
-                tm_wait_ld(xm_, x0_, x1_);
-            }
+            tm_ld(cx(0), xm_);
+            tm_ld(cx(1), x0_);
+            tm_ld(cx(2), x1_);
+            tm_wait_ld(xm_, x0_, x1_);
             tm_st(cx(3), x2_);
             dstar_z2<EW>(P0, P1, x0_, x1_, x2_, xm_, e, lb, rb, m2.cA[2], m2.cD[2], m2.cB[2][0],
                       m2.cB[2][1], dz2);
@@ -365,16 +350,10 @@ step_kernel(const __grid_constant__ FusedMaps maps, Geom g, Mult<float> m, Mult2
             // B_z = B_z + (D*_y E_x - D*_x E_y)
             dstar_y2<EW>(Pm, P0, P1, x0_, x1_, xm_, e, lb, rb, m2.cA[1], m2.cD[1], m2.cB[1][0],
                       m2.cB[1][2], dy2);
-            if (it == 0) {
-                ym_ = ldq(Pm + ESLOT, e);
-                y0_ = ldq(P0 + ESLOT, e);
-                y1_ = ldq(P1 + ESLOT, e);
-            } else {
-                tm_ld(cy(0), ym_);
-                tm_ld(cy(1), y0_);
-                tm_ld(cy(2), y1_);
-                tm_wait_ld(ym_, y0_, y1_);
-            }
+            tm_ld(cy(0), ym_);
+            tm_ld(cy(1), y0_);
+            tm_ld(cy(2), y1_);
+            tm_wait_ld(ym_, y0_, y1_);
             dstar_x4<EW>(Pm + ESLOT, P0 + ESLOT, P1 + ESLOT, y0_, y1_, ym_, e, lb, rb, m.cA[0],
                      m.cD[0], m.cB[0][1], m.cB[0][2], t);
 #pragma unroll
