@@ -25,7 +25,8 @@
 //     cost nothing.
 // 256^3 points: 3350 us with the printed formulas, 1315 us here (floor of 42 FP64 instructions a
 // point on that pipe: 1220 us); 30 degree cone 1446 -> 237 us; 256^2 points, launch-bound, 46 us in
-// three kernels -> 22 us in two.
+// three kernels -> 19 us in two (2 us of it the blocks' sums, 3 us the last block's: 7 us when it
+// read the partials one quantity after another).
 // A thread takes one row segment at a time, neighbouring threads neighbouring k_y; a block's sums
 // are taken once, and the block that arrives last adds the blocks' partials in a fixed order
 // (deterministic result).
@@ -131,12 +132,21 @@ __device__ __forceinline__ double norm_block_sum(const double (&v)[NQ], double (
 #pragma unroll
     for (int q = 0; q < NQ; ++q) sm[q][threadIdx.x] = v[q];
     __syncthreads();
+    constexpr int WARPS = NORM_BLOCK / 32, R = (NQ + WARPS - 1) / WARPS;
     const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-    for (int q = w; q < NQ; q += NORM_BLOCK / 32) {
-        double x = (sm[q][l] + sm[q][l + 32]) + (sm[q][l + 64] + sm[q][l + 96]);
-        for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
-        if (l == 0) res[q] = x;
+    double x[R];   // the warp's quantities together: independent chains of FP64 additions
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const int q = min(w + r * WARPS, NQ - 1);
+        x[r] = (sm[q][l] + sm[q][l + 32]) + (sm[q][l + 64] + sm[q][l + 96]);
     }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+        for (int r = 0; r < R; ++r) x[r] += __shfl_down_sync(0xffffffffu, x[r], o);
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+        if (l == 0 && w + r * WARPS < NQ) res[w + r * WARPS] = x[r];
     __syncthreads();
     return threadIdx.x < NQ ? res[threadIdx.x] : 0.0;
 }
@@ -258,11 +268,11 @@ norm_kernel(NormParams p, const double2* __restrict__ tab, const Angle* __restri
     if (!last) return;
     __threadfence();
 #pragma unroll
-    for (int q = 0; q < NQ; ++q) {
-        acc[q] = 0.0;
-        for (unsigned b = threadIdx.x; b < gridDim.x; b += NORM_BLOCK)
+    for (int q = 0; q < NQ; ++q) acc[q] = 0.0;
+    for (unsigned b = threadIdx.x; b < gridDim.x; b += NORM_BLOCK)
+#pragma unroll
+        for (int q = 0; q < NQ; ++q)   // the quantities' loads in flight together
             acc[q] += __ldcg(part + (long long)q * gridDim.x + b);
-    }
     const double total = norm_block_sum(acc, sm, res);
     // out[14] = {f, dbeta 3x3 row-major, ddelta 3, ddt}
     const int slot[NQ] = {0, 1 + 1, 1 + 2, 1 + 3, 1 + 5, 1 + 6, 1 + 7, 10, 11, 12, 13};
@@ -343,14 +353,16 @@ static void fill_params(NormParams& p, const double alpha[3], const double beta[
 }
 
 // Runs the two kernels on `st` using `scratch` (norm_scratch_doubles() doubles);
-// the 14 results land in scratch's last 16 entries and are returned via *out_dev.
+// the 14 results land at host_out (device address of pinned host memory) or, if that is NULL, in
+// scratch's last 16 entries, returned via *out_dev.
 // Segment length: one warp a scheduler (152 x 4 x 32 threads) saturates the FP64 pipe, so few
 // points are cut into that many segments of at least 4 (256^2 points: 17.4 us with 4, 22 with 2,
 // 35 with 16), many into segments of 64 (256^3: 1284 us, 16: 1310); of 16 with the cone weight, whose
 // rows differ in work (231 us, 64: 295).
 void launch_disp_norm(const double alpha[3], const double beta[3][3], const double delta[3],
                       double dt, const double dx[3], int dims, const int N[3], int weight,
-                      double wparam, double* scratch, double** out_dev, cudaStream_t st) {
+                      double wparam, double* scratch, double* host_out, double** out_dev,
+                      cudaStream_t st) {
     NormParams p;
     fill_params(p, alpha, beta, delta, dt, dx, dims, N, weight, wparam);
     const long long per = (p.npts + 152 * 128 - 1) / (152 * 128);
@@ -367,6 +379,9 @@ void launch_disp_norm(const double alpha[3], const double beta[3][3], const doub
     norm_table_kernel<<<(unsigned)((entries + 63) / 64), 64, 0, st>>>(p, dx[0], dx[1], dx[2], tab, ang,
                                                                       ticket);
     const int nb = (int)std::min<long long>((items + NORM_BLOCK - 1) / NORM_BLOCK, NORM_GRID);
+    if (host_out != nullptr) out = host_out;
+    // (no dependent launch: blocks placed while the table's still run share the SMs unevenly, a whole
+    // call of the cone 252 -> 302 us, of 256^3 1330 -> 1337 to 1617, against 1.5 us gained on 256^2)
     norm_kernel<<<nb, NORM_BLOCK, 0, st>>>(p, tab, ang, part, ticket, out);
     *out_dev = out;
 }
@@ -558,7 +573,8 @@ size_t group_scratch_doubles(const int N[3], long long npts) {
 
 void launch_disp_group_norm(const double alpha[3], const double beta[3][3], const double delta[3],
                             double dt, const double dx[3], int dims, const int N[3], int weight,
-                            double wparam, double* scratch, double** out_dev, cudaStream_t st) {
+                            double wparam, double* scratch, double* host_out, double** out_dev,
+                            cudaStream_t st) {
     GroupParams gp;
     NormParams& p = gp.n;
     fill_params(p, alpha, beta, delta, dt, dx, dims, N, weight, wparam);
@@ -572,6 +588,7 @@ void launch_disp_group_norm(const double alpha[3], const double beta[3][3], cons
     if (p.N[2] > nmax) nmax = p.N[2];
     group_table_kernel<<<(nmax + 255) / 256, 256, 0, st>>>(gp, tab);
     group_norm_kernel<<<nb, NORM_THREADS, 0, st>>>(gp, tab, part);
+    if (host_out != nullptr) out = host_out;
     norm_final_kernel<<<1, dim3(32, NQ), 0, st>>>(part, nb, p.pref, out);
     *out_dev = out;
 }
