@@ -615,8 +615,14 @@ bool adjoint32f_supported(const Geom& g) {
            g.ny >= adj32f::TY && g.total < (1LL << 31);
 }
 
+bool adjoint2d32_prepare();
+void launch_adjoint2d32(const FusedMaps&, const Geom&, const Mult<float>&, FieldSet<float>,
+                        const float* const[3], const float*, const float*, double*, int, int, int*,
+                        cudaStream_t);
+
 bool adjoint32f_prepare() {
-    return cudaFuncSetAttribute(adj32f::adjF_kernel<true>,
+    return adjoint2d32_prepare() &&
+           cudaFuncSetAttribute(adj32f::adjF_kernel<true>,
                                 cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)adj32f::SMEM) == cudaSuccess &&
            cudaFuncSetAttribute(adj32f::adjF_kernel<false>,
@@ -642,11 +648,17 @@ int adjoint32f_blocks(const Geom& g) {
 
 // maps.e[c]: 72 x 12 boxes of lambda_E component c of the input set `lam`, maps.b[c]: 72 x 11
 // boxes of its lambda_B component c; E: the forward
-// E^n of the step (padded arrays); the result goes to `out` (the other set)
+// E^n of the step (padded arrays); the result goes to `out` (the other set).  Planes that do not
+// couple along z (flat) take the kernel without halo planes (fdtd_adjoint2d.cu), same results
 void launch_adjoint32_fused(const FusedMaps& maps, const Geom& g, const Mult<float>& m,
                             FieldSet<float> lam, FieldSet<float> out, const float* const E[3],
-                            const float* spy, const float* spz, double* partials, int* err,
-                            cudaStream_t st) {
+                            const float* spy, const float* spz, double* partials, bool flat,
+                            int* err, cudaStream_t st) {
+    if (flat) {
+        launch_adjoint2d32(maps, g, m, out, E, spy, spz, partials, adjoint32f_tz(g),
+                           adjoint32f_blocks(g), err, st);
+        return;
+    }
     auto kern = spy != nullptr ? adj32f::adjF_kernel<true> : adj32f::adjF_kernel<false>;
     launch_pdl(kern, dim3((unsigned)adjoint32f_blocks(g)), dim3(adj32f::NT), adj32f::SMEM, st, maps, g, m,
                lam, out, E[0], E[1], E[2], spy, spz, partials, adjoint32f_tz(g), err);

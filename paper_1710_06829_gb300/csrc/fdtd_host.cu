@@ -65,7 +65,7 @@ bool adjoint32f_prepare();
 int adjoint32f_blocks(const Geom& g);
 void launch_adjoint32_fused(const FusedMaps& maps, const Geom& g, const Mult<float>& m,
                             FieldSet<float> lam, FieldSet<float> out, const float* const E[3],
-                            const float* spy, const float* spz, double* partials, int* err,
+                            const float* spy, const float* spz, double* partials, bool flat, int* err,
                             cudaStream_t st);
 void launch_adjoint32_E(const FusedMaps& maps, const Geom& g, const Mult<float>& m,
                         FieldSet<float> lam, const float* spy, const float* spz, int* err,
@@ -1019,7 +1019,7 @@ static int adjoint_impl(fdtd_handle* h, int n, const fdtd_probe* probe, double* 
                 FieldSet<float> nxt;
                 for (int c = 0; c < 6; ++c) nxt.c[c] = (float*)h->lam_arr_set(h->lam_cur ^ 1, c);
                 launch_adjoint32_fused(h->lam_emaps[h->lam_cur], g, m, lam, nxt, E, spy, spz,
-                                       h->partials, h->err_dev, h->stream);
+                                       h->partials, h->plan->flat, h->err_dev, h->stream);
                 CK(cudaGetLastError());
                 h->lam_cur ^= 1;
                 continue;

@@ -325,3 +325,35 @@ def test_fp64_reverse_step_matches_the_reference_form(shape, sponge, monkeypatch
     for a, b in zip(out[0][0], out[1][0]):
         assert float((a - b).abs().max()) <= 1e-13 * max(float(c.abs().max()) for c in out[1][0])
     assert float((out[0][1] - out[1][1]).abs().max()) <= 1e-11 * float(out[1][1].abs().max())
+
+
+@pytest.mark.parametrize("shape,dims,kw", [
+    ((64, 8, 1), 2, {}), ((64, 16, 1), 3, {}), ((128, 24, 2), 2, dict(batched=True)),
+    ((192, 8, 17), 2, dict(batched=True)), ((64, 40, 70), 2, dict(batched=True)),
+    ((128, 16, 9), 2, dict(batched=True, absorb_cells=3, absorb_sigma=0.3))])
+def test_fp32_reverse_step_of_planes_matches_fp64(shape, dims, kw, monkeypatch):
+    """lambda and the gradient of three recorded steps, with a probe on the last column, against the
+    FP64 reference form on the same FP32 inputs.  Per value about 20 FP32 operations a step on terms
+    of the field's size, forward and back: 6 x 20 x 2^-24 = 7e-6 of the largest value, 2e-5 taken;
+    the gradient's terms carry that error with random signs, like the terms themselves: 1e-4 of
+    the largest entry."""
+    from paper_1710_06829_gb300 import sim as S
+    f = [torch.from_numpy(a) for a in _random_state(shape, "f32", 14)]
+    lam = [torch.from_numpy(a) for a in _random_state(shape, "f32", 15)]
+    nx, ny, nz = shape
+    tgt = torch.from_numpy(np.random.default_rng(4).standard_normal((3, nz, ny)).astype(np.float32)).cuda()
+    out = []
+    for flag, dtype, tt in (("1", "f32", torch.float32), ("0", "f64", torch.float64)):
+        monkeypatch.setenv("FDTD_FUSED", flag)
+        sm = _sim(shape, dtype, dims=dims, **kw)
+        sm.set_state([t.to(tt) for t in f])
+        sm.step(3, record=True)
+        sm.set_adjoint([t.to(tt) for t in lam])
+        grad = torch.zeros(12, dtype=torch.float64, device="cuda")
+        sm.step_adjoint(3, grad, probe=S.Probe(1, nx - 1, tgt.to(tt)))
+        out.append(([t.double() for t in sm.get_adjoint()], grad.cpu()))
+        sm.sync()
+        sm.close()
+    for a, b in zip(out[0][0], out[1][0]):
+        assert float((a - b).abs().max()) <= 2e-5 * max(float(c.abs().max()) for c in out[1][0])
+    assert float((out[0][1] - out[1][1]).abs().max()) <= 1e-4 * float(out[1][1].abs().max())
