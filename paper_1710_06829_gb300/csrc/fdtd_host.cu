@@ -1229,9 +1229,11 @@ static int check_species(const fdtd_handle* h, const fdtd_species* sp, int32_t n
     return FDTD_OK;
 }
 
+template <typename T>
 static bool ensure_bmean(fdtd_handle* h) {
     if (h->bmean) return true;
-    if (cudaMalloc(&h->bmean, (size_t)3 * h->g.total * h->esz) == cudaSuccess) return true;
+    if (pic_mean_prepare<T>() &&
+        cudaMalloc(&h->bmean, (size_t)3 * h->g.total * h->esz) == cudaSuccess) return true;
     h->bmean = nullptr;
     (void)cudaGetLastError();
     return false;
@@ -1251,11 +1253,11 @@ static int pic_impl(fdtd_handle* h, int n, const fdtd_species* sp, int nsp) {
     // B^n once per cell (a pass of 36 B a cell in FP32) where the particles save more by it (24 of
     // 72 loads each); without the memory for it, once per particle.  Us a cycle, per particle / per
     // cell, particles drifted by a cell: 128^3 and 0.5 per cell 183 / 177, 1 per cell 277 / 255, 2 per
-    // cell 461 / 401; 64^3 and 1 per cell 62 / 63, 2 per cell 83 / 80.
+    // cell 461 / 401; 64^3 and 1 per cell 62 / 63, 2 per cell 83 / 80 (per cell now 4 to 6 % less).
     const long long cells = (long long)g.nx * g.ny * g.nz;
     long long np = 0;
     for (int q = 0; q < nsp; ++q) np += sp[q].n;
-    const bool mean = n > 0 && np >= cells && np >= (1 << 20) && ensure_bmean(h);
+    const bool mean = n > 0 && np >= cells && np >= (1 << 20) && ensure_bmean<T>(h);
     for (int s = 0; s < n; ++s) {
         FieldSet<T> cur = fieldset<T>(h, h->cur), nxt = fieldset<T>(h, 1 - h->cur);
         // (E^{n+1} without the current, B^{n+1/2}) into the other set: Ampere's law is linear

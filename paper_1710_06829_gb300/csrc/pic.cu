@@ -35,7 +35,7 @@
 //   - where all 32 particles of a warp sit in one cell (a dense bunch, particles kept in cell
 //     order), the values of each face are summed through shared memory and added once.
 // Push per cycle: bunch of 2^22 particles in a 512 x 256 x 256 grid 717 -> 214 us; 2^22 particles of
-// a 128^3 plasma, drifted by a cell, 823 -> 317 us (332 with single additions instead of add_pair),
+// a 128^3 plasma, drifted by a cell, 823 -> 287 us (with single additions instead of add_pair 15 us more),
 // bound by L2 (72 % busy: 10 sectors of additions and 11 of loads a particle) and L1 (76 %).
 #include <climits>
 #include <cmath>
@@ -305,19 +305,31 @@ __device__ __forceinline__ void deposit_shared(T* __restrict__ E, const Move<T, 
     }
 }
 
+// Threads of a block: with particles all over the grid (MEAN) one block fills an SM, so that the
+// 24 warps of a sweep read neighbouring field rows and the next sweep finds them in L1 (plasma
+// 317 us with three blocks of 256, 287 with one of 768; in cell order no difference); a bunch is spread over more, smaller
+// blocks, whose work differs less (214 us with nine of 256 an SM, 234 to 254 with blocks of 768).
+// FP64 is bound by its pipe either way (3585 and 3600 us a cycle).
+template <typename T, bool MEAN>
+constexpr int PUSH = MEAN && sizeof(T) == 4 ? 3 * THREADS : THREADS;
+template <typename T, bool MEAN>
+constexpr size_t PUSH_SMEM = (size_t)(PUSH<T, MEAN> / 32) * 18 * ROW * sizeof(T);
+
 // MEAN: a.B0 holds B^n; otherwise B^n = (B0 + B1) / 2 per node.  SP: absorbing layers.  I: type of the
 // element offsets (int where a padded array has fewer than 2^31 elements).
 template <typename T, bool MEAN, bool SP, typename I>
-__global__ void __launch_bounds__(THREADS, sizeof(T) == 4 ? 3 : 2) push_kernel(PushArgs<T> a) {
+__global__ void __launch_bounds__(PUSH<T, MEAN>, sizeof(T) == 8 ? 2 : MEAN ? 1 : 3)
+push_kernel(PushArgs<T> a) {
     const Geom& g = a.g;
-    __shared__ __align__(16) T rows[THREADS / 32][18 * ROW];
+    extern __shared__ __align__(16) unsigned char smem[];
+    T (*rows)[18 * ROW] = reinterpret_cast<T (*)[18 * ROW]>(smem);   // of each warp
     const I Y = (I)g.nxp, Z = (I)g.plane;
     // A block takes a contiguous range of particles: with particles in about the order of their cells
-    // it then finds the field rows of one sweep of 256 in L1 for the next (bunch: 214 us, in
+    // it then finds the field rows of one sweep in L1 for the next (bunch: 214 us, in
     // interleaved sweeps 260).  The loop bound is block-uniform, so every lane runs every iteration.
     const long long per = ((a.n + gridDim.x - 1) / gridDim.x + 31) / 32 * 32;
     const long long first = blockIdx.x * per, end = first + per < a.n ? first + per : a.n;
-    for (long long base = first; base < end; base += THREADS) {
+    for (long long base = first; base < end; base += PUSH<T, MEAN>) {
         const long long p = base + threadIdx.x;
         bool live = p < end;
         T x = 0, y = 0, z = 0, ux = 0, uy = 0, uz = 0;
@@ -520,12 +532,28 @@ inline unsigned blocks_for(long long n) {
 }  // namespace picd
 
 template <typename T>
+bool pic_mean_prepare() {
+    auto set = [](auto kern) {
+        return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)picd::PUSH_SMEM<T, true>) == cudaSuccess;
+    };
+    return set(picd::push_kernel<T, true, true, int>) && set(picd::push_kernel<T, true, false, int>) &&
+           set(picd::push_kernel<T, true, true, long long>) &&
+           set(picd::push_kernel<T, true, false, long long>);
+}
+template bool pic_mean_prepare<float>();
+template bool pic_mean_prepare<double>();
+
+template <typename T>
 void launch_pic_push(const PushArgs<T>& a, bool mean, cudaStream_t st) {
     if (a.n <= 0) return;
-    // nine blocks an SM (three resident; 456, 912, 1368, 4864 blocks: bunch 227, 217, 214, 237 us)
-    const long long want = (a.n + picd::THREADS - 1) / picd::THREADS;
-    const unsigned blocks = (unsigned)(want < 9 * 152 ? want : 9 * 152);
-    auto go = [&](auto kern) { kern<<<blocks, picd::THREADS, 0, st>>>(a); };
+    // nine blocks of 256 an SM (three resident; 456, 912, 1368, 4864 blocks: bunch 227, 217, 214, 237
+    // us) or one large one (1, 2, 3, 6 an SM: plasma 287, 291, 295, 308 us)
+    const int threads = mean ? picd::PUSH<T, true> : picd::PUSH<T, false>;
+    const size_t smem = mean ? picd::PUSH_SMEM<T, true> : picd::PUSH_SMEM<T, false>;
+    const long long want = (a.n + threads - 1) / threads, most = (threads > picd::THREADS ? 1 : 9) * 152;
+    const unsigned blocks = (unsigned)(want < most ? want : most);
+    auto go = [&](auto kern) { kern<<<blocks, threads, smem, st>>>(a); };
     const bool sp = a.spy != nullptr;
     auto with = [&](auto idx) {
         using I = decltype(idx);

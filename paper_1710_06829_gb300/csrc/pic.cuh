@@ -45,7 +45,9 @@ struct PushArgs {
     T escale[3];   // q / (dx_b dx_c): the cumulative shape change of axis a times this is -dt J_a
     int* err;
 };
-// mean: B0 holds B^n itself (launch_bmean) and B1 is not read.
+// mean: B0 holds B^n itself (launch_bmean) and B1 is not read; pic_mean_prepare first.
+template <typename T>
+bool pic_mean_prepare();
 template <typename T>
 void launch_pic_push(const PushArgs<T>& a, bool mean, cudaStream_t st);
 

@@ -357,3 +357,47 @@ def test_fp32_reverse_step_of_planes_matches_fp64(shape, dims, kw, monkeypatch):
     for a, b in zip(out[0][0], out[1][0]):
         assert float((a - b).abs().max()) <= 2e-5 * max(float(c.abs().max()) for c in out[1][0])
     assert float((out[0][1] - out[1][1]).abs().max()) <= 1e-4 * float(out[1][1].abs().max())
+
+
+@pytest.mark.parametrize("sponge", [False, True])
+@pytest.mark.parametrize("n", [1 << 20, (1 << 20) + 77])
+def test_push_of_many_particles_matches_that_of_few(n, sponge):
+    """1000 charged particles alone, and beside n neutral ones that only drift: the second call takes
+    the push for many particles (B once per cell, one large block an SM).  Positions of up to 32 cells
+    differ by a few units of 2^-19 cells (B's rounding, three cycles); a deposit of charge 0.01 by as
+    much of it, far below 1e-5 of fields of 0.3."""
+    from paper_1710_06829_gb300 import inputs
+    from paper_1710_06829_gb300 import sim as S
+    shape = (32, 12, 16)
+    rng = np.random.default_rng(8)
+    ext = np.array(shape)[:, None]
+    def species(m, q, qm):
+        x = (rng.uniform(0, 0.999, (3, m)) * ext).astype(np.float32)
+        u = rng.standard_normal((3, m)).astype(np.float32)
+        return x, u, q, qm
+    few, many = species(1000, 0.01, -1.0), species(n, 0.0, 0.0)
+    f = [torch.from_numpy(0.1 * a).float() for a in inputs.random_fields(shape, 7)]
+    out = []
+    for sps in ([few], [few, many]):
+        sm = _sim(shape, "f32", **(dict(absorb_cells=2, absorb_sigma=0.3) if sponge else {}))
+        sm.set_state(f)
+        sp = [S.Species(torch.from_numpy(x.copy()).cuda(), torch.from_numpy(u.copy()).cuda(), q, qm)
+              for x, u, q, qm in sps]
+        sm.pic_step(3, sp)
+        sm.sync()
+        out.append((sm.get_state(), sp))
+        sm.close()
+    big = max(float(t.abs().max()) for t in out[0][0])
+    for a, b in zip(out[0][0], out[1][0]):
+        assert float((a - b).abs().max()) <= 1e-5 * big
+    L = torch.tensor(shape, dtype=torch.float64, device="cuda")[:, None]
+
+    def far(a, b):   # a position on the seam may sit at either end
+        d = (a.double() - b.double()).abs()
+        return float(torch.minimum(d, L - d).max())
+    a, b = out[0][1][0], out[1][1][0]
+    assert far(a.x, b.x) <= 1e-4 and float((a.u - b.u).abs().max()) <= 1e-5 * float(a.u.abs().max())
+    x, u = (torch.from_numpy(v).double().cuda() for v in many[:2])
+    assert torch.equal(out[1][1][1].u, torch.from_numpy(many[1]).cuda())
+    x = torch.remainder(x + 3 * 0.4 * u / torch.sqrt(1 + (u * u).sum(0)), L)
+    assert far(out[1][1][1].x, x) <= 1e-4
