@@ -245,6 +245,7 @@ __global__ void reduce_grad_kernel(const double* __restrict__ part, int nblocks,
     const int q = threadIdx.y;       // 0..8
     const int l = threadIdx.x;       // 0..31
     double v = 0.0;
+#pragma unroll 8
     for (int b = l; b < nblocks; b += 32) v += part[(long long)b * 9 + q];
     red[q][l] = v;
     __syncthreads();

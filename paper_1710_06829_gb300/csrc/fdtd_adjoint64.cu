@@ -18,6 +18,9 @@ namespace adj64 {
 using namespace seg64;
 
 constexpr int NT = 128;
+// of a lambda block: single warps, as in the forward step (us a reverse step with blocks of 128 / 32:
+// 60 x 32 x 39 37.3 / 27.1, 64^3 69.5 / 62.4, 192 x 128 x 96 472 / 474)
+constexpr int NL = 32;
 
 template <bool SP>
 __global__ void __launch_bounds__(NT)
@@ -189,13 +192,13 @@ __device__ __forceinline__ void dt_z(const double* G2, const double* Gm, const d
 
 // SP: absorbing layers.  partials[block][9] += (delta_a, beta_a,b1, beta_a,b2) for a = x, y, z
 template <bool SP>
-__global__ void __launch_bounds__(NT, 2)
+__global__ void __launch_bounds__(NL, 2 * NT / NL)
 lambda_kernel(Geom g, Mult<double> m, FieldSet<double> lam, const double* __restrict__ e_x,
               const double* __restrict__ e_y, const double* __restrict__ e_z,
               const double* __restrict__ spy, const double* __restrict__ spz,
               double* __restrict__ partials, int tz) {
     pdl_wait();
-    const Tile t = tile_of(g, (long long)blockIdx.x * NT + threadIdx.x);
+    const Tile t = tile_of(g, (long long)blockIdx.x * NL + threadIdx.x);
     const int z0 = blockIdx.y * tz, zend = min(z0 + tz, g.nz);
     double acc[3][4];   // per axis: sums of w (far pair, first, second transverse sum, difference)
 #pragma unroll
@@ -283,28 +286,30 @@ lambda_kernel(Geom g, Mult<double> m, FieldSet<double> lam, const double* __rest
         }
     }
     pdl_trigger();
-    // block sums, one warp a quantity at a time
-    __shared__ double sm[9][NT];
+    // the warp's sums: lane 3 q + r adds every third value of quantity q, the first of three the rest
+    __shared__ double sm[9][NL + 1];
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
         sm[3 * a][threadIdx.x] = fma(-3.0, acc[a][3], acc[a][0]);
         sm[3 * a + 1][threadIdx.x] = fma(-2.0, acc[a][3], acc[a][1]);
         sm[3 * a + 2][threadIdx.x] = fma(-2.0, acc[a][3], acc[a][2]);
     }
-    __syncthreads();
-    const int wp = threadIdx.x >> 5, l = threadIdx.x & 31;
-    for (int q = wp; q < 9; q += NT / 32) {
-        double x = (sm[q][l] + sm[q][l + 32]) + (sm[q][l + 64] + sm[q][l + 96]);
-        for (int s = 16; s > 0; s >>= 1) x += __shfl_down_sync(0xffffffffu, x, s);
-        if (l == 0) partials[((long long)blockIdx.y * gridDim.x + blockIdx.x) * 9 + q] += x;
+    __syncwarp();
+    const int l = threadIdx.x, q = l / 3;
+    double x = 0.0;
+    if (q < 9) {
+        for (int k = l % 3; k < NL; k += 3) x += sm[q][k];
     }
+    const double x1 = __shfl_down_sync(0xffffffffu, x, 1), x2 = __shfl_down_sync(0xffffffffu, x, 2);
+    if (q < 9 && l % 3 == 0)
+        partials[((long long)blockIdx.y * gridDim.x + blockIdx.x) * 9 + q] += x + (x1 + x2);
 }
 
 }  // namespace adj64
 
 static dim3 adjoint64_grid(const Geom& g, int& tz) {
-    tz = march64(g, adj64::NT);
-    const long long columns = (seg64::tiles(g) + adj64::NT - 1) / adj64::NT;
+    tz = march64(g, adj64::NL);
+    const long long columns = (seg64::tiles(g) + adj64::NL - 1) / adj64::NL;
     return dim3((unsigned)columns, (unsigned)((g.nz + tz - 1) / tz));
 }
 
@@ -322,7 +327,7 @@ void launch_adjoint64(const Geom& g, const Mult<double>& m, FieldSet<double> lam
     launch_pdl(spy ? mu_kernel<true> : mu_kernel<false>, dim3(nb), dim3(NT), 0, st, g, m, lam, spy, spz);
     int tz;
     const dim3 grid = adjoint64_grid(g, tz);
-    launch_pdl(spy ? lambda_kernel<true> : lambda_kernel<false>, grid, dim3(NT), 0, st, g, m, lam, E[0],
+    launch_pdl(spy ? lambda_kernel<true> : lambda_kernel<false>, grid, dim3(NL), 0, st, g, m, lam, E[0],
                E[1], E[2], spy, spz, partials, tz);
 }
 

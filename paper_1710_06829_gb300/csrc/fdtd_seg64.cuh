@@ -192,9 +192,8 @@ __device__ __forceinline__ void dstar_z(const double* Fm, const double* F0, cons
 }  // namespace seg64
 
 // Planes a thread of the marching FP64 kernels takes, blocks of `threads` threads: the FP64 pipe is
-// the limit, so the SM with the most blocks decides, blocks x (planes + the first plane's extra
-// differences, a quarter of a plane's work); a single block an SM leaves its schedulers one warp
-// each and takes 1.3 times its share.
+// the limit, so the scheduler with the most warps decides, warps x (planes + the first plane's extra
+// differences, a quarter of a plane's work); a single warp takes 1.3 times its share.
 int march64(const Geom& g, int threads);
 
 }  // namespace fdtd

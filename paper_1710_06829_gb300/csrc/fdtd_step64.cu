@@ -9,7 +9,8 @@
 // come from L1.  About 77 FP64 instructions a cell and step, where the reference form takes 99.
 // Values and rounding order are those of dstar_diff / ampere_comp: bitwise the same fields.
 // Us a step, the kernels before (one tiled kernel with barriers where 64 x 8 tiles fit, else the
-// reference form) and these: 192 x 128 x 96 717 / 385, 100 x 90 x 80 199 / 127, 36^3 27 / 18,
+// reference form) and these: 192 x 128 x 96 717 / 385, 100 x 90 x 80 199 / 124, 36^3 27 / 18,
+// 60 x 32 x 39 31 / 19,
 // 128^3 638 / 331 (0.157 ns a cell, 91 issue slots of the FP64 pipe).  A kernel that shares every
 // difference through shared memory (76 instructions, two barriers a plane) took 518 us at
 // 192 x 128 x 96: the pipe idles at the barriers.
@@ -23,14 +24,19 @@ namespace step64 {
 using namespace seg64;
 
 constexpr int NT = 128;
+// Threads of a Faraday block.  A warp's plane takes 8 us of its scheduler, so a small grid is a
+// question of how evenly its warps fall on the SMs: single warps do best (us a step with blocks of
+// 128, 64, 32: 60 x 32 x 39 27.8, 22.6, 18.6; 48^3 29.0, 24.5, 24.4; 64^3 52.8, 53.0, 48.0; 192 x 128 x
+// 96 384.6, 385.0, 384.8).
+constexpr int NF = 32;
 
 // SP: absorbing layers
 template <bool SP>
-__global__ void __launch_bounds__(NT, 3)
+__global__ void __launch_bounds__(NF, 3 * NT / NF)
 faraday_kernel(Geom g, Mult<double> m, FieldSet<double> in, FieldSet<double> out,
                const double* __restrict__ spy, const double* __restrict__ spz, int tz) {
     pdl_wait();
-    const Tile t = tile_of(g, blockIdx.x * NT + threadIdx.x);
+    const Tile t = tile_of(g, (long long)blockIdx.x * NF + threadIdx.x);
     const int z0 = blockIdx.y * tz, zend = min(z0 + tz, g.nz);
     if (t.j < 0) return;
     const double *Ex = in.c[0] + t.o, *Ey = in.c[1] + t.o, *Ez = in.c[2] + t.o;
@@ -157,9 +163,9 @@ int march64(const Geom& g, int threads) {
     int best = 1;
     double best_cost = -1.0;
     for (int tz = g.nz < 64 ? g.nz : 64; tz >= 1; --tz) {
-        const long long blocks = columns * ((g.nz + tz - 1) / tz);
-        const double per_sm = (double)((blocks + 151) / 152);
-        const double cost = (per_sm > 1.0 ? per_sm : 1.3) * (tz + 0.25);
+        const long long blocks = columns * ((g.nz + tz - 1) / tz), per_sm = (blocks + 151) / 152;
+        const double warps = (double)((per_sm * (threads / 32) + 3) / 4);   // of the fullest scheduler
+        const double cost = (warps > 1.0 ? warps : 1.3) * (tz + 0.25);
         if (best_cost < 0.0 || cost < best_cost) {
             best_cost = cost;
             best = tz;
@@ -172,10 +178,10 @@ void launch_step64(const Geom& g, const Mult<double>& m, FieldSet<double> in, Fi
                    const double* spy, const double* spz, const double* jyz, const double* jx_row,
                    double* hist_E[3], int* err, cudaStream_t st) {
     using namespace step64;
-    const int tz = march64(g, NT);
+    const int tz = march64(g, NF);
     const long long tiles = seg64::tiles(g);
-    const dim3 grid((unsigned)((tiles + NT - 1) / NT), (unsigned)((g.nz + tz - 1) / tz));
-    launch_pdl(spy ? faraday_kernel<true> : faraday_kernel<false>, grid, dim3(NT), 0, st, g, m, in, out,
+    const dim3 grid((unsigned)((tiles + NF - 1) / NF), (unsigned)((g.nz + tz - 1) / tz));
+    launch_pdl(spy ? faraday_kernel<true> : faraday_kernel<false>, grid, dim3(NF), 0, st, g, m, in, out,
                spy, spz, tz);
     const long long pairs = (long long)(g.nx / 2) * g.ny * g.nz;
     const unsigned nb = (unsigned)std::min<long long>((pairs + NT - 1) / NT, 1 << 20);
