@@ -1,9 +1,14 @@
 // FP32 fused leapfrog step (one launch per leapfrog step).
 //
+// Bound: issue and latency at 14 warps an SM, next to HBM (48 B a cell).  Us a step, before ragged
+// tiles, the schedule's chunk lengths, the specialisations and the rows filled before the march, and
+// now: 256^3 180 / 166.5 (805 MB: 0.71 of the copy rate), 128^3 39 / 28, 64^3 35 / 10, 300 x 250 x 225
+// with layers and a bunch (two reference-form kernels before) 440 / 187.
+//
 // A CTA owns a 64 x 8 (x, y) tile and a chunk of tz planes (a launch parameter) and marches
-// through it; the last tiles of a ragged grid reach past its cells and drop what they form there.  E^n planes arrive by TMA (cp.async.bulk.tensor.3d) as 76 x 12 boxes (x0-4 ..,
-// y0-2 ..) into a ring of five shared-memory slots, one plane ahead of use, completion signalled
-// on mbarriers.  Iteration `it` forms B^{n+1/2} on plane p = z0-1+it (tile, halo row y0-1, halo
+// through it; the last tiles of a ragged grid reach past its cells and drop what they form there.
+// E^n planes arrive by TMA (cp.async.bulk.tensor.3d) as 76 x 12 boxes (x0-4 .., y0-2 ..) into a ring
+// of five shared-memory slots, one plane ahead of use, completion signalled on mbarriers.  Iteration `it` forms B^{n+1/2} on plane p = z0-1+it (tile, halo row y0-1, halo
 // column x0-1) and E^{n+1} on plane p-1, so one block barrier per plane suffices; B^{n+1/2}
 // lives in a small shared ring (B_x, B_y: 3 planes, B_z: 2 planes).  B^{n-1/2} is not staged:
 // each thread prefetches its own segment of the next plane from HBM into registers while the
@@ -630,8 +635,6 @@ static int fused32_tz(const Geom& g) {
     using namespace f32seg;
     static int slots = -1;
     if (slots < 0) slots = resident_slots_tmem((const void*)step_kernel<false, false>, NT, SMEM, TM_COLS);
-    // measured at 256^3 (456 resident CTAs): 37-plane chunks (2 full waves) 0.218 ms per step,
-    // 32-plane chunks (2.25 waves) 0.269 ms
     return zchunk_len(tiles32(g), g.nz, slots, 2, 64);
 }
 
