@@ -13,7 +13,9 @@
 //   d/d beta_ab:  [(F[+a+b] - F[+b]) + (F[+a-b] - F[-b]) - 2 (F[+a] - F[0])] / dx_a
 // Kernel adjB computes mu (written to lambda_B) and the gradient partials;
 // kernel adjE then updates lambda_E from the new lambda_B.
-#include "fdtd_internal.cuh"
+#include <type_traits>
+
+#include "fdtd_seg.cuh"
 
 namespace fdtd {
 
@@ -219,9 +221,139 @@ void launch_adjoint_B_v0(const Geom& g, const Mult<T>& m, FieldSet<T> lam, const
                                                         sponge_y, sponge_z, partials);
 }
 
+// The same for FP32, four cells of a row a thread: 29 16-byte loads and 22 of one value, instead of 300
+// of one value, the differences that the cells share formed once.  Values and order are those
+// of dstarT_at.  Bound: L1 and L2 (every row comes to each block that reads it).  Us, one cell a
+// thread and this kernel: 300 x 250 x 56 75.6 / 46.5, 140 x 100 x 150 41.1 / 22.3, 100 x 90 x 80
+// 15.8 / 10.2, 500 x 300 x 32 78.5 / 52.3, 36^3 4.3 / 4.5.  At 300 x 250 x 56 tiles of several rows a
+// block take 58, the stores at the end 51.4.
+__global__ void __launch_bounds__(128)
+adjoint_E4_kernel(Geom g, Mult<float> m, FieldSet<float> lam, const float* __restrict__ spy,
+                  const float* __restrict__ spz, int n) {
+    using namespace seg;
+    const int t = blockIdx.x * 128 + threadIdx.x, ns = g.nx / 4;
+    if (t >= n) return;
+    const int row = t / ns, i = (t - row * ns) * 4, k = row / g.ny, j = row - k * g.ny;
+    const int c = (int)pidx(g, i, j, k), Y = g.nxp;
+    const int zp = (int)zoff_a(g, k, 1), zm = (int)zoff_a(g, k, -1), zmm = (int)zoff_a(g, k, -2);
+    const float *X = lam.c[3] + c, *V = lam.c[4] + c, *Z = lam.c[5] + c;
+    // DT along an axis of one component: the own row o, one back b, two back bb, one ahead f of the
+    // row, and the differences b - o of the rows beside (p, q: first axis, r, s: second)
+    auto comb = [](const float* d, const float* bb, const float* f, const float* p, const float* q,
+                   const float* r, const float* s, float cA, float cD, float cB, float cC, float* out) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            float v = cA * d[u];
+            v = fma(cD, bb[u] - f[u], v);
+            v = fma(cB, p[u] + q[u], v);
+            out[u] = fma(cC, r[u] + s[u], v);
+        }
+    };
+    auto diff = [](const Q4& a, const Q4& b, float* d) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) d[u] = a.v[u] - b.v[u];
+    };
+    // differences of one row against the next along x, x-1 .. x+4's: transverse x neighbours of d
+    auto beside = [](const float* d, float lo, float hi, float* left, float* right) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            left[u] = u ? d[u ? u - 1 : 0] : lo;
+            right[u] = u < 3 ? d[u < 3 ? u + 1 : 3] : hi;
+        }
+    };
+    // differences along x of a row whose value at x-1 is l
+    auto along = [](float l, const Q4& a, float* d) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) d[u] = (u ? a.v[u ? u - 1 : 0] : l) - a.v[u];
+    };
+    // DT_x: own row a (x-2, x-1, x+4 in l2, l1, r), rows y-1, y+1, z-1, z+1 with their values at x-1
+    auto dtx = [&](const Q4& a, float l2, float l1, float r, const Q4& ym, float lym, const Q4& yp,
+                   float lyp, const Q4& bm, float lbm, const Q4& bp, float lbp, float* out) {
+        float d[4], p[4], q[4], e[4], f[4], bb[4], ff[4];
+        along(l1, a, d);
+        along(lym, ym, p);
+        along(lyp, yp, q);
+        along(lbm, bm, e);
+        along(lbp, bp, f);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            bb[u] = u == 0 ? l2 : u == 1 ? l1 : a.v[u > 1 ? u - 2 : 0];
+            ff[u] = u < 3 ? a.v[u < 3 ? u + 1 : 3] : r;
+        }
+        comb(d, bb, ff, p, q, e, f, m.cA[0], m.cD[0], m.cB[0][1], m.cB[0][2], out);
+    };
+    // DT_y of the component at G: own rows a (y), b (y-1), f (y+1); values beside the own row at
+    // x-1 and x+4 in al, ar; rows (y, z-1), (y, z+1) in am, ap
+    auto dty = [&](const float* G, const Q4& a, const Q4& b, const Q4& f, float al, float ar, const Q4& am,
+                   const Q4& bm, const Q4& ap, float* out) {
+        const Q4 bb = ldq(G, -2 * Y), bp = ldq(G, zp - Y);
+        float d[4], l[4], r[4], e[4], h[4];
+        diff(b, a, d);
+        beside(d, G[-Y - 1] - al, G[-Y + 4] - ar, l, r);
+        diff(bm, am, e);
+        diff(bp, ap, h);
+        comb(d, bb.v, f.v, l, r, e, h, m.cA[1], m.cD[1], m.cB[1][0], m.cB[1][2], out);
+    };
+    // DT_z: own rows a (z), b (z-1), f (z+1); beside a and b at x-1, x+4 in al, ar, bl, br; rows y-1
+    // and y+1 of z in am, ap, of z-1 in bm, bp
+    auto dtz = [&](const float* G, const Q4& a, const Q4& b, const Q4& f, float al, float ar, float bl,
+                   float br, const Q4& am, const Q4& bm, const Q4& ap, const Q4& bp, float* out) {
+        const Q4 bb = ldq(G, zmm);
+        float d[4], l[4], r[4], e[4], h[4];
+        diff(b, a, d);
+        beside(d, bl - al, br - ar, l, r);
+        diff(bm, am, e);
+        diff(bp, ap, h);
+        comb(d, bb.v, f.v, l, r, e, h, m.cA[2], m.cD[2], m.cB[2][0], m.cB[2][1], out);
+    };
+    const float s0 = sp_at(g, spy, spz, j, k);
+    const bool edge = i < PX || i >= g.nx - PX || j < PY || j >= g.ny - PY;
+    const SegOut dst = seg_out(g, i, j, edge);
+    const unsigned po = (unsigned)k * (unsigned)g.plane;
+    auto put = [&](int q, const float* a, const float* b) {
+        const Q4 l = ldq(lam.c[q], c);
+        float v[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) v[u] = __fmaf_rn(s0, l.v[u], __fsub_rn(a[u], b[u]));
+        put_seg(lam.c[q], po, dst, v);
+    };
+    float yz[4], xz[4], zy[4], xy[4], zx[4], yx[4];
+    {   // mu_z: DT_y, DT_x
+        const Q4 a = ldq(Z, 0), b = ldq(Z, -Y), f = ldq(Z, Y), am = ldq(Z, zm), ap = ldq(Z, zp),
+                 bm = ldq(Z, zm - Y);
+        const float l1 = Z[-1], r = Z[4];
+        dty(Z, a, b, f, l1, r, am, bm, ap, yz);
+        dtx(a, Z[-2], l1, r, b, Z[-Y - 1], f, Z[Y - 1], am, Z[zm - 1], ap, Z[zp - 1], xz);
+    }
+    {   // mu_y: DT_z, DT_x
+        const Q4 a = ldq(V, 0), b = ldq(V, zm), f = ldq(V, zp), am = ldq(V, -Y), ap = ldq(V, Y);
+        const float l1 = V[-1], r = V[4], bl = V[zm - 1];
+        dtz(V, a, b, f, l1, r, bl, V[zm + 4], am, ldq(V, zm - Y), ap, ldq(V, zm + Y), zy);
+        dtx(a, V[-2], l1, r, am, V[-Y - 1], ap, V[Y - 1], b, bl, f, V[zp - 1], xy);
+    }
+    put(0, yz, zy);
+    {   // mu_x: DT_z, DT_y
+        const Q4 a = ldq(X, 0), b = ldq(X, zm), f = ldq(X, zp), am = ldq(X, -Y), ap = ldq(X, Y),
+                 bm = ldq(X, zm - Y);
+        const float l1 = X[-1], r = X[4];
+        dtz(X, a, b, f, l1, r, X[zm - 1], X[zm + 4], am, bm, ap, ldq(X, zm + Y), zx);
+        dty(X, a, am, ap, l1, r, b, bm, f, yx);
+    }
+    put(1, zx, xz);
+    put(2, xy, yx);
+}
+
 template <typename T>
 void launch_adjoint_E_v0(const Geom& g, const Mult<T>& m, FieldSet<T> lam, const T* sponge_y,
                          const T* sponge_z, cudaStream_t st) {
+    if constexpr (std::is_same<T, float>::value) {
+        // put_seg's single image offsets want nx >= 8 and ny >= 4, the kernel 32-bit offsets
+        if (g.nx >= 2 * PX && g.ny >= 2 * PY && g.total < (1LL << 31)) {
+            const int n = g.nx / 4 * g.ny * g.nz;
+            adjoint_E4_kernel<<<(n + 127) / 128, 128, 0, st>>>(g, m, lam, sponge_y, sponge_z, n);
+            return;
+        }
+    }
     dim3 blk(128), grd((g.nx + 127) / 128, (unsigned)(g.ny < 65535 ? g.ny : 65535),
                         (unsigned)(g.nz < 65535 ? g.nz : 65535));   // j, k loop in the kernel
     adjoint_E_kernel<T><<<grd, blk, 0, st>>>(g, m, lam, sponge_y, sponge_z);

@@ -401,3 +401,12 @@ def test_push_of_many_particles_matches_that_of_few(n, sponge):
     assert torch.equal(out[1][1][1].u, torch.from_numpy(many[1]).cuda())
     x = torch.remainder(x + 3 * 0.4 * u / torch.sqrt(1 + (u * u).sum(0)), L)
     assert far(out[1][1][1].x, x) <= 1e-4
+
+
+@pytest.mark.parametrize("shape,dims,kw", [
+    ((8, 4, 1), 3, {}), ((8, 5, 2), 3, {}), ((12, 9, 3), 3, {}), ((68, 33, 21), 3, {}),
+    ((132, 7, 5), 2, dict(batched=True)), ((36, 20, 30), 3, dict(absorb_cells=4, absorb_sigma=0.3))])
+def test_fp32_reverse_step_of_ragged_grids_matches_fp64(shape, dims, kw, monkeypatch):
+    """As above, on grids without whole tiles: down to the smallest that the kernel of four cells a
+    thread takes, one to three planes, layers."""
+    test_fp32_reverse_step_of_planes_matches_fp64(shape, dims, kw, monkeypatch)
