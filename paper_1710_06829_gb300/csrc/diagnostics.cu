@@ -104,8 +104,8 @@ energy_kernel(Geom g, FieldSet<T> s, int x_lo, int x_len, int my, int mz, double
 // (the former kernel), 6.1 us here.
 template <typename T>
 __global__ void __launch_bounds__(DG_THREADS)
-probe_loss_kernel(Geom g, const T* __restrict__ F, int xp, const T* __restrict__ target,
-                  double* part, unsigned* ticket, double* loss) {
+probe_loss_kernel(Geom g, const T* F, int xp, const T* target, double* part, unsigned* ticket,
+                  double* loss) {
     pdl_trigger();
     pdl_wait();
     double acc[1] = {0.0};
@@ -207,7 +207,7 @@ __global__ void phase_kernel(Geom g, double kx, double ky, double kz, double ox,
 
 template <typename T>
 __global__ void __launch_bounds__(DG_THREADS)
-planewave_kernel(Geom g, const T* __restrict__ F, const double2* __restrict__ tab, double* part,
+planewave_kernel(Geom g, const T* F, const double2* tab, double* part,
                  unsigned* ticket, double* out) {
     constexpr int V = Vec<T>::N;
     pdl_trigger();

@@ -18,7 +18,7 @@
 // compensated FP32 sum a thread and axis), so lambda and the gradient are bitwise those of that kernel.
 //
 // Bound: HBM for a large batch (60 B a cell), launch and latency for a small one.  Us a step, the 3D
-// kernel and this one: 512 x 512 x 32 148 / 102 (503 MB: 0.73 of the copy rate), 512 x 512 x 8 50 / 29,
+// kernel and this one: 512 x 512 x 32 148 / 97 (503 MB: 0.76 of the copy rate), 512 x 512 x 8 50 / 29,
 // 1024 x 1024 72 / 27, 192 x 40 x 70 38 / 23, 64 x 8 8.7 / 4.3.
 #include "fdtd_seg.cuh"
 
@@ -110,8 +110,7 @@ __device__ __forceinline__ void dtx(const float* G, const float* R, int e, bool 
 template <bool SP>
 __global__ void __launch_bounds__(NT, 4)
 adj2d_kernel(const __grid_constant__ FusedMaps maps, Geom g, Mult<float> m, FieldSet<float> out,
-             const float* __restrict__ e_x, const float* __restrict__ e_y,
-             const float* __restrict__ e_z, const float* __restrict__ spy,
+             const float* e_x, const float* e_y, const float* e_z, const float* __restrict__ spy,
              const float* __restrict__ spz, double* __restrict__ partials, int tz,
              int* __restrict__ err) {
     extern __shared__ __align__(128) unsigned char smem[];
@@ -228,9 +227,9 @@ adj2d_kernel(const __grid_constant__ FusedMaps maps, Geom g, Mult<float> m, Fiel
         const int q = z0 + it;
         const unsigned po = (unsigned)q * plane;
         float eo[3][W];   // E^n of the own cells, used after the barrier
-        unpackv(__ldg(reinterpret_cast<const float4*>(e_x + po + dst.ro)), eo[0]);
-        unpackv(__ldg(reinterpret_cast<const float4*>(e_y + po + dst.ro)), eo[1]);
-        unpackv(__ldg(reinterpret_cast<const float4*>(e_z + po + dst.ro)), eo[2]);
+        unpackv(__ldcg(reinterpret_cast<const float4*>(e_x + po + dst.ro)), eo[0]);
+        unpackv(__ldcg(reinterpret_cast<const float4*>(e_y + po + dst.ro)), eo[1]);
+        unpackv(__ldcg(reinterpret_cast<const float4*>(e_z + po + dst.ro)), eo[2]);
         const float* L = sL + (it % NL) * 3 * LSLOT;
         float* M = sM + mslot * 3 * MSLOT;
         float mu[3][W], le[3][W];

@@ -189,9 +189,8 @@ __device__ __forceinline__ void dtx_g(const float* Gm, const float* G0, const fl
 template <bool SP>
 __global__ void __launch_bounds__(NT, 2)
 adjF_kernel(const __grid_constant__ FusedMaps maps, Geom g, Mult<float> m, FieldSet<float> lam,
-            FieldSet<float> out, const float* __restrict__ e_x, const float* __restrict__ e_y,
-            const float* __restrict__ e_z, const float* __restrict__ spy,
-            const float* __restrict__ spz, double* __restrict__ partials, int tz,
+            FieldSet<float> out, const float* e_x, const float* e_y, const float* e_z,
+            const float* __restrict__ spy, const float* __restrict__ spz, double* __restrict__ partials, int tz,
             int* __restrict__ err) {
     extern __shared__ __align__(128) unsigned char smem[];
     float* sL = reinterpret_cast<float*>(smem);
@@ -322,8 +321,8 @@ adjF_kernel(const __grid_constant__ FusedMaps maps, Geom g, Mult<float> m, Field
     const float* ea1 = grp1 ? e_z : e_y;
     auto load_e = [&](int qw, float (&to)[2][W]) {
         const unsigned off = (unsigned)qw * plane + dst.ro;
-        unpackv(__ldg(reinterpret_cast<const float4*>(ea0 + off)), to[0]);
-        unpackv(__ldg(reinterpret_cast<const float4*>(ea1 + off)), to[1]);
+        unpackv(*reinterpret_cast<const float4*>(ea0 + off), to[0]);
+        unpackv(*reinterpret_cast<const float4*>(ea1 + off), to[1]);
     };
     load_e(wrapz(z0), en);
 

@@ -37,18 +37,14 @@ mu_kernel(Geom g, Mult<double> m, FieldSet<double> lam, const double* __restrict
         ld2(lam.c[0] + o, ex);
         ld2(lam.c[1] + o, ey);
         ld2(lam.c[2] + o, ez);
-        ey[2] = __ldg(lam.c[1] + o + 2);
-        ez[2] = __ldg(lam.c[2] + o + 2);
+        ey[2] = lam.c[1][o + 2];
+        ez[2] = lam.c[2][o + 2];
         ld2(lam.c[0] + o + Y, exy);
         ld2(lam.c[2] + o + Y, ezy);
         ld2(lam.c[0] + oz, exz);
         ld2(lam.c[1] + oz, eyz);
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {   // read and written here: no read-only load
-            const double2 v = *reinterpret_cast<const double2*>(lam.c[3 + c] + o);
-            b[c][0] = v.x;
-            b[c][1] = v.y;
-        }
+        for (int c = 0; c < 3; ++c) ld2(lam.c[3 + c] + o, b[c]);
         double s0 = 1.0, sy = 1.0, sz = 1.0;
         if (SP) {
             s0 = spy[j] * spz[k];
@@ -83,7 +79,7 @@ __device__ __forceinline__ void own_tx(const double* G, long long Y, Quad& d) {
     for (int r = 0; r < 2; ++r) {
         double a[2];
         ld2(G + r * Y, a);
-        const double b = __ldg(G + r * Y - 1);
+        const double b = G[r * Y - 1];
         d.v[r][0] = b - a[0];
         d.v[r][1] = a[0] - a[1];
     }
@@ -116,17 +112,17 @@ __device__ __forceinline__ void dt_x(const double* G, long long Y, const Quad& d
                                      const Quad& w, double* acc, Quad& out) {
     double lo[2], hi[2], a[2];   // rows y-1, y+2
     ld2(G - Y, a);
-    lo[0] = __ldg(G - Y - 1) - a[0];
+    lo[0] = G[-Y - 1] - a[0];
     lo[1] = a[0] - a[1];
     ld2(G + 2 * Y, a);
-    hi[0] = __ldg(G + 2 * Y - 1) - a[0];
+    hi[0] = G[2 * Y - 1] - a[0];
     hi[1] = a[0] - a[1];
 #pragma unroll
     for (int r = 0; r < 2; ++r) {
         const double* q = G + r * Y;
         double lf[2];   // x-2, x-1
         ld2(q - 2, lf);
-        const double r1 = __ldg(q + 1), r2 = __ldg(q + 2);
+        const double r1 = q[1], r2 = q[2];
 #pragma unroll
         for (int u = 0; u < 2; ++u)
             out.v[r][u] = dt_value(d0.v[r][u], lf[u] - (u ? r2 : r1),
@@ -141,8 +137,8 @@ __device__ __forceinline__ void dt_y(const double* G, long long Y, const Quad& d
                                      const Quad& w, double* acc, Quad& out) {
 #pragma unroll
     for (int r = 0; r < 2; ++r) {
-        const double lf = __ldg(G + (r - 1) * Y - 1) - __ldg(G + r * Y - 1);
-        const double rt = __ldg(G + (r - 1) * Y + 2) - __ldg(G + r * Y + 2);
+        const double lf = G[(r - 1) * Y - 1] - G[r * Y - 1];
+        const double rt = G[(r - 1) * Y + 2] - G[r * Y + 2];
         double dn[2], up[2];   // rows y-2, y+1
         ld2(G + (r - 2) * Y, dn);
         ld2(G + (r + 1) * Y, up);
@@ -166,8 +162,8 @@ __device__ __forceinline__ void dt_z(const double* G2, const double* Gm, const d
         ld2(G0 + r * Y, b);
 #pragma unroll
         for (int u = 0; u < 2; ++u) d.v[r][u] = a[u] - b[u];
-        lf[r] = __ldg(Gm + r * Y - 1) - __ldg(G0 + r * Y - 1);
-        rt[r] = __ldg(Gm + r * Y + 2) - __ldg(G0 + r * Y + 2);
+        lf[r] = Gm[r * Y - 1] - G0[r * Y - 1];
+        rt[r] = Gm[r * Y + 2] - G0[r * Y + 2];
     }
     ld2(Gm - Y, a);
     ld2(G0 - Y, b);
@@ -193,9 +189,8 @@ __device__ __forceinline__ void dt_z(const double* G2, const double* Gm, const d
 // SP: absorbing layers.  partials[block][9] += (delta_a, beta_a,b1, beta_a,b2) for a = x, y, z
 template <bool SP>
 __global__ void __launch_bounds__(NL, 2 * NT / NL)
-lambda_kernel(Geom g, Mult<double> m, FieldSet<double> lam, const double* __restrict__ e_x,
-              const double* __restrict__ e_y, const double* __restrict__ e_z,
-              const double* __restrict__ spy, const double* __restrict__ spz,
+lambda_kernel(Geom g, Mult<double> m, FieldSet<double> lam, const double* e_x, const double* e_y,
+              const double* e_z, const double* __restrict__ spy, const double* __restrict__ spz,
               double* __restrict__ partials, int tz) {
     pdl_wait();
     const Tile t = tile_of(g, (long long)blockIdx.x * NL + threadIdx.x);
@@ -241,8 +236,8 @@ lambda_kernel(Geom g, Mult<double> m, FieldSet<double> lam, const double* __rest
 #pragma unroll
                 for (int r = 0; r < 2; ++r) {
                     if (r && !t.two) break;
-                    const double2 l = *reinterpret_cast<const double2*>(lam.c[c] + t.o + o0 + r * Y);
-                    double v[2] = {l.x, l.y};
+                    double v[2];
+                    ld2(lam.c[c] + t.o + o0 + r * Y, v);
 #pragma unroll
                     for (int u = 0; u < 2; ++u) {
                         const double d = a.v[r][u] - b.v[r][u];

@@ -98,7 +98,7 @@ template <bool SP, bool JX>
 __global__ void __launch_bounds__(NT, 3)
 step_kernel(const __grid_constant__ FusedMaps maps, Geom g, Mult<float> m, Mult2 m2, FieldSet<float> in,
             FieldSet<float> out, const float* __restrict__ spy, const float* __restrict__ spz,
-            const float* __restrict__ jyz, const float* __restrict__ jx_row,
+            const float* __restrict__ jyz, const float* jx_row,
             float* __restrict__ h0, float* __restrict__ h1, float* __restrict__ h2, int zs, int ze,
             int tz, int* __restrict__ err) {
     extern __shared__ __align__(128) unsigned char smem[];
@@ -220,7 +220,7 @@ step_kernel(const __grid_constant__ FusedMaps maps, Geom g, Mult<float> m, Mult2
         const unsigned o = (unsigned)qw * plane + b_off;
 #pragma unroll
         for (int c = 0; c < 3; ++c)
-            unpackv(__ldg(reinterpret_cast<const float4*>(in.c[3 + c] + o)), to[c]);
+            unpackv(*reinterpret_cast<const float4*>(in.c[3 + c] + o), to[c]);
     };
     load_bold(wrapz(z0 - 1), bn);
 
@@ -232,7 +232,7 @@ step_kernel(const __grid_constant__ FusedMaps maps, Geom g, Mult<float> m, Mult2
         sp_n = spz[wrapz(z0 - 1)];
     }
     if (JX) {
-        unpackv(__ldg(reinterpret_cast<const float4*>(jx_row + max(b_i, 0))), jv);
+        unpackv(*reinterpret_cast<const float4*>(jx_row + max(b_i, 0)), jv);
         const float sy = jyz[max(b_j, 0)];
 #pragma unroll
         for (int u = 0; u < W; ++u) jv[u] *= sy;

@@ -51,7 +51,7 @@ __device__ __forceinline__ bool nonfinite(double v) {
 }
 
 __device__ __forceinline__ void ld2(const double* p, double* v) {
-    const double2 a = __ldg(reinterpret_cast<const double2*>(p));
+    const double2 a = *reinterpret_cast<const double2*>(p);
     v[0] = a.x;
     v[1] = a.y;
 }
@@ -79,7 +79,7 @@ __device__ __forceinline__ void own_dx(const double* F, long long Y, Quad& d) {
     for (int r = 0; r < 2; ++r) {
         double a[2];
         ld2(F + r * Y, a);
-        const double b = __ldg(F + r * Y + 2);
+        const double b = F[r * Y + 2];
         d.v[r][0] = a[1] - a[0];
         d.v[r][1] = b - a[1];
     }
@@ -104,11 +104,11 @@ __device__ __forceinline__ void dstar_x(const double* F, long long Y, const Quad
     {
         double a[2];
         ld2(F - Y, a);
-        const double b = __ldg(F - Y + 2);
+        const double b = F[-Y + 2];
         lo[0] = a[1] - a[0];
         lo[1] = b - a[1];
         ld2(F + 2 * Y, a);
-        const double c = __ldg(F + 2 * Y + 2);
+        const double c = F[2 * Y + 2];
         hi[0] = a[1] - a[0];
         hi[1] = c - a[1];
     }
@@ -118,7 +118,7 @@ __device__ __forceinline__ void dstar_x(const double* F, long long Y, const Quad
         double mid[2], rt[2];
         ld2(q, mid);
         ld2(q + 2, rt);
-        const double lf = __ldg(q - 1);
+        const double lf = q[-1];
 #pragma unroll
         for (int u = 0; u < 2; ++u)
             out.v[r][u] = dstar_diff(d0.v[r][u], rt[u], u ? mid[0] : lf, r ? hi[u] : d0.v[1][u],
@@ -134,8 +134,8 @@ __device__ __forceinline__ void dstar_y(const double* F, long long Y, long long 
     double lf[2], rt[2];   // y differences of columns x-1, x+2
 #pragma unroll
     for (int r = 0; r < 2; ++r) {
-        lf[r] = __ldg(F + (r + 1) * Y - 1) - __ldg(F + r * Y - 1);
-        rt[r] = __ldg(F + (r + 1) * Y + 2) - __ldg(F + r * Y + 2);
+        lf[r] = F[(r + 1) * Y - 1] - F[r * Y - 1];
+        rt[r] = F[(r + 1) * Y + 2] - F[r * Y + 2];
     }
 #pragma unroll
     for (int r = 0; r < 2; ++r) {
@@ -162,8 +162,8 @@ __device__ __forceinline__ void dstar_z(const double* Fm, const double* F0, cons
         ld2(F0 + r * Y, b);
 #pragma unroll
         for (int u = 0; u < 2; ++u) d.v[r][u] = a[u] - b[u];
-        lf[r] = __ldg(F1 + r * Y - 1) - __ldg(F0 + r * Y - 1);
-        rt[r] = __ldg(F1 + r * Y + 2) - __ldg(F0 + r * Y + 2);
+        lf[r] = F1[r * Y - 1] - F0[r * Y - 1];
+        rt[r] = F1[r * Y + 2] - F0[r * Y + 2];
     }
     {
         double a[2], b[2];

@@ -506,8 +506,7 @@ template void launch_pack<double>(const Geom&, const double* const[6], double* c
 
 // lambda_E[x_p, j, k] += 2 (F[x_p, j, k] - T[k][j]), written with its periodic images.
 template <typename T>
-__global__ void probe_adjoint_kernel(Geom g, T* __restrict__ lam, const T* __restrict__ F, int xp,
-                                     const T* __restrict__ target) {
+__global__ void probe_adjoint_kernel(Geom g, T* lam, const T* F, int xp, const T* target) {
     pdl_trigger();
     pdl_wait();
     const int t = blockIdx.x * blockDim.x + threadIdx.x;

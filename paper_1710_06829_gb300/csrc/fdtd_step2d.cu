@@ -15,7 +15,7 @@
 //
 // Bound: launch and latency for a small plane, HBM and L2 for a large batch.  Us a step, the 3D kernel (whole tiles) or
 // the reference form before and this kernel: 128 x 128 33 / 2.8 (4.2 without the dependent launch),
-// 1000 x 750 24 / 7.9 (10.3), 512 x 512 x 32 107 / 77 (80; 805 MB: 0.77 of the copy rate).
+// 1000 x 750 24 / 8.0 (10.3), 512 x 512 x 32 107 / 76 (403 MB: 0.78 of the copy rate).
 #include "fdtd_seg.cuh"
 
 namespace fdtd {
@@ -38,7 +38,7 @@ __device__ __forceinline__ void copy16(float* dst, const float* src) {
 __global__ void __launch_bounds__(NT)
 step2d_kernel(Geom g, Mult<float> m, Mult2 m2, FieldSet<float> in, FieldSet<float> out,
               const float* __restrict__ spy, const float* __restrict__ spz,
-              const float* __restrict__ jyz, const float* __restrict__ jx_row,
+              const float* __restrict__ jyz, const float* jx_row,
               float* __restrict__ h0, float* __restrict__ h1, float* __restrict__ h2,
               int* __restrict__ err) {
     __shared__ __align__(16) float sE[3 * EPL];
@@ -54,18 +54,6 @@ step2d_kernel(Geom g, Mult<float> m, Mult2 m2, FieldSet<float> in, FieldSet<floa
     const unsigned plane = (unsigned)g.plane, po = (unsigned)k * plane;
     const bool edge = (x0 < PX) || (x0 + TX > g.nx - PX) || (y0 < PY) || (y0 + TY > g.ny - PY);
 
-    // E box: padded row y0 + r and column x0 + 4 c hold (x0-4+4c, y0-2+r); a ragged tile's box stops
-    // at the ghosts
-    const int rows = min(EH, g.nyp - y0), cols = min(EW, g.nxp - x0) / W;
-    for (int t = tid; t < EH * (EW / W); t += NT) {
-        const int r = t / (EW / W), c = t - r * (EW / W);
-        if (r >= rows || c >= cols) continue;
-        const unsigned o = po + (unsigned)((y0 + r) * g.nxp + x0 + W * c);
-#pragma unroll
-        for (int q = 0; q < 3; ++q) copy16(sE + q * EPL + r * EW + W * c, in.c[q] + o);
-    }
-    asm volatile("cp.async.commit_group;" ::: "memory");
-
     // task of this thread, as in the 3D kernel: owned rows, then the halo row y0-1, then the halo
     // column (its segment's last cell x0-1 is the one that is used), then idle copies of the last
     const int bx = tid < NSEG * (TY + 1) ? W * (tid % NSEG) : -W;
@@ -77,11 +65,23 @@ step2d_kernel(Geom g, Mult<float> m, Mult2 m2, FieldSet<float> in, FieldSet<floa
     const bool lb = bx == 0, rb = bx < 0 || bx == TX - W;
     const int e = (by + 2) * EW + (bx + 4), bi = (by + 1) * BW + (bx + 4);
     const SegOut dst = seg_out(g, max(i, 0), max(j, 0), edge);
-    float bo[3][W];
+    float bo[3][W];   // before the box's copies (behind them: 512 x 512 x 32 80 us, here 76)
 #pragma unroll
     for (int c = 0; c < 3; ++c)
-        unpackv(__ldg(reinterpret_cast<const float4*>(in.c[3 + c] + po +
-                                                      (unsigned)((j + PY) * g.nxp + i + PX))), bo[c]);
+        unpackv(*reinterpret_cast<const float4*>(in.c[3 + c] + po + (unsigned)((j + PY) * g.nxp + i + PX)),
+                bo[c]);
+
+    // E box: padded row y0 + r and column x0 + 4 c hold (x0-4+4c, y0-2+r); a ragged tile's box stops
+    // at the ghosts
+    const int rows = min(EH, g.nyp - y0), cols = min(EW, g.nxp - x0) / W;
+    for (int t = tid; t < EH * (EW / W); t += NT) {
+        const int r = t / (EW / W), c = t - r * (EW / W);
+        if (r >= rows || c >= cols) continue;
+        const unsigned o = po + (unsigned)((y0 + r) * g.nxp + x0 + W * c);
+#pragma unroll
+        for (int q = 0; q < 3; ++q) copy16(sE + q * EPL + r * EW + W * c, in.c[q] + o);
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
     float f = 1.0f;
     if (spy != nullptr) f = spy[j < 0 ? j + g.ny : j] * spz[k];
 
@@ -147,7 +147,7 @@ step2d_kernel(Geom g, Mult<float> m, Mult2 m2, FieldSet<float> in, FieldSet<floa
     if (!live) return;
     if (jx_row != nullptr) {
         float jv[W];
-        unpackv(__ldg(reinterpret_cast<const float4*>(jx_row + i)), jv);
+        unpackv(*reinterpret_cast<const float4*>(jx_row + i), jv);
         const float sy = jyz[j], sz = jyz[g.ny + k];
 #pragma unroll
         for (int u = 0; u < W; ++u) ex[u] = fma(-m.dt, (jv[u] * sy) * sz, ex[u]);

@@ -39,7 +39,7 @@ template <int TX, int TY, bool ZC>
 __global__ void __launch_bounds__(TX* TY)
 step2d64_kernel(Geom g, Mult<double> m, FieldSet<double> in, FieldSet<double> out,
                 const double* __restrict__ spy, const double* __restrict__ spz,
-                const double* __restrict__ jyz, const double* __restrict__ jx_row,
+                const double* __restrict__ jyz, const double* jx_row,
                 double* __restrict__ h0, double* __restrict__ h1, double* __restrict__ h2,
                 int* __restrict__ err) {
     using C = Cfg<TX, TY>;
@@ -76,7 +76,7 @@ step2d64_kernel(Geom g, Mult<double> m, FieldSet<double> in, FieldSet<double> ou
         const int i = min(x0 - 1 + c, g.nx - 1), j = min(y0 - 1 + r, g.ny - 1);
         const long long o = po + (long long)(j + PY) * g.nxp + (i + PX);
 #pragma unroll
-        for (int a = 0; a < 3; ++a) b[q][a] = __ldg(in.c[3 + a] + o);
+        for (int a = 0; a < 3; ++a) b[q][a] = in.c[3 + a][o];
     }
     asm volatile("cp.async.wait_group 0;" ::: "memory");
     __syncthreads();

@@ -110,7 +110,7 @@ template <bool SP>
 __global__ void __launch_bounds__(NT)
 ampere_kernel(Geom g, Mult<double> m, FieldSet<double> in, FieldSet<double> out,
               const double* __restrict__ spy, const double* __restrict__ spz,
-              const double* __restrict__ jyz, const double* __restrict__ jx_row,
+              const double* __restrict__ jyz, const double* jx_row,
               double* __restrict__ h0, double* __restrict__ h1, double* __restrict__ h2,
               int* __restrict__ err) {
     pdl_wait();
@@ -131,7 +131,7 @@ ampere_kernel(Geom g, Mult<double> m, FieldSet<double> in, FieldSet<double> out,
         ld2(Bz + o - Y, bzy);
         ld2(Bx + om, bxz);
         ld2(By + om, byz);
-        const double byl = __ldg(By + o - 1), bzl = __ldg(Bz + o - 1);
+        const double byl = By[o - 1], bzl = Bz[o - 1];
         const double f = SP ? spy[j] * spz[k] : 1.0;
 #pragma unroll
         for (int u = 0; u < 2; ++u) {

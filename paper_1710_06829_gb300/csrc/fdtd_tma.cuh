@@ -26,6 +26,14 @@ struct FusedPlan {
 // pdl_trigger() or ended, and pdl_wait() returns when that kernel has completed and its writes are
 // visible.  A kernel launched this way calls pdl_wait() in every thread before it touches global
 // memory.  Between the steps of a time loop this hides about 2 us of launch latency.
+//
+// Such a kernel is resident while the kernels before it still write, so what an earlier kernel of
+// the stream may have written (fields, adjoint fields, recorded E, phase tables, the bunch table,
+// probe targets) is read after pdl_wait() with plain loads or __ldcg, through pointers that are not
+// const __restrict__: __ldg, and what the compiler makes of const __restrict__, ask for data that
+// does not change during the kernel's life, may be moved above the wait and may be served from
+// lines that an earlier kernel left in L1.  Only the layers' factors and the bunch's transverse
+// profile, complete before the host queues the first step, are read that way.
 template <class... P, class... A>
 inline void launch_pdl(void (*k)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... a) {
     cudaLaunchConfig_t cfg = {};

@@ -1,0 +1,84 @@
+"""Calls queued one behind the other without a synchronisation, as programs queue them, against the
+same calls with the device idle before each: small grids, so that the kernels of several calls are
+resident at once (dependent launches).  Everything is deterministic: the results are equal bit by bit."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+pytestmark = pytest.mark.gpu
+
+# the FP32 3D march, the FP64 3D pair of kernels, one plane and a batch in either precision
+GRIDS = [((64, 16, 8), 3, "f32", {}), ((20, 12, 6), 3, "f32", dict(absorb_cells=2, absorb_sigma=0.3)),
+         ((20, 12, 6), 3, "f64", {}), ((128, 48, 1), 2, "f32", {}), ((64, 24, 3), 2, "f32", dict(batched=True)),
+         ((48, 40, 1), 2, "f64", {}), ((16, 9, 4), 2, "f64", dict(batched=True))]
+
+
+def _runs(shape, dims, dtype, kw, body):
+    """body(simulation, between) with nothing and with a synchronisation between its calls"""
+    from paper_1710_06829_gb300 import inputs
+    from paper_1710_06829_gb300 import sim as S
+    beta, delta = inputs.isotropic_theta(-0.05, -0.04, 0.02, 0.01)
+    f = [torch.from_numpy(a) for a in inputs.random_fields(shape, 31)]
+    out = []
+    for between in (lambda: None, torch.cuda.synchronize):
+        sm = S.Simulation(shape, [1.0, 1.0, 1.0], 0.4, beta, delta, dims=dims, dtype=dtype, **kw)
+        sm.set_state(f)
+        out.append(body(sm, between))
+        sm.sync()
+        sm.close()
+    return out
+
+
+@pytest.mark.parametrize("shape,dims,dtype,kw", GRIDS)
+def test_plane_waves_of_different_k_and_steps(shape, dims, dtype, kw):
+    rng = np.random.default_rng(5)
+    calls = [(int(rng.integers(6)), tuple(rng.uniform(-3, 3, 3))) for _ in range(24)]
+
+    def body(sm, between):
+        res = torch.zeros((len(calls), 2), dtype=torch.float64, device="cuda")
+        torch.cuda.synchronize()
+        for n, (comp, k) in enumerate(calls):
+            sm.plane_wave(comp, k, out=res[n])
+            between()
+            if n % 3 == 2:
+                sm.step(1)
+                between()
+        torch.cuda.synchronize()
+        return res
+    a, b = _runs(shape, dims, dtype, kw, body)
+    assert torch.equal(a, b) and bool((a != 0).any())
+
+
+@pytest.mark.parametrize("shape,dims,dtype,kw", GRIDS)
+def test_steps_probes_and_reverse_steps(shape, dims, dtype, kw):
+    from paper_1710_06829_gb300 import sim as S
+    nx, ny, nz = shape
+    tt = torch.float32 if dtype == "f32" else torch.float64
+    n = 24
+    tgt = torch.from_numpy(np.random.default_rng(6).standard_normal((n + 4, nz, ny))).to(tt).cuda()
+
+    def body(sm, between):
+        loss = torch.zeros(1, dtype=torch.float64, device="cuda")
+        grad = torch.zeros(12, dtype=torch.float64, device="cuda")
+        probe = S.Probe(1, nx - 1, tgt)
+        src = None if kw.get("batched") else S.Bunch(1.0, 0.9, 3.0, 2.0, 1.0, 2.0, 2.0)
+        sm.set_adjoint()
+        torch.cuda.synchronize()
+        for _ in range(n // 2):
+            sm.step(1, source=src)
+            between()
+        for _ in range(n // 2):
+            sm.step(1, probe=probe, loss=loss)
+            between()
+        state = sm.get_state()
+        sm.step(4, record=True)
+        between()
+        for _ in range(4):
+            sm.step_adjoint(1, grad, probe=probe)
+            between()
+        return [*state, *sm.get_adjoint(), loss, grad]
+    a, b = _runs(shape, dims, dtype, kw, body)
+    for x, y in zip(a, b):
+        assert torch.equal(x, y)
+    assert float(a[12]) > 0 and float(a[13].abs().max()) > 0
