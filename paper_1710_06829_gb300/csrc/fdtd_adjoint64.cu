@@ -191,10 +191,11 @@ template <bool SP>
 __global__ void __launch_bounds__(NL, 2 * NT / NL)
 lambda_kernel(Geom g, Mult<double> m, FieldSet<double> lam, const double* e_x, const double* e_y,
               const double* e_z, const double* __restrict__ spy, const double* __restrict__ spz,
-              double* __restrict__ partials, int tz) {
+              double* __restrict__ partials, int tz, unsigned columns) {
     pdl_wait();
-    const Tile t = tile_of(g, (long long)blockIdx.x * NL + threadIdx.x);
-    const int z0 = blockIdx.y * tz, zend = min(z0 + tz, g.nz);
+    const unsigned chunk = blockIdx.x / columns, column = blockIdx.x - chunk * columns;
+    const Tile t = tile_of(g, (long long)column * NL + threadIdx.x);
+    const int z0 = (int)chunk * tz, zend = min(z0 + tz, g.nz);
     double acc[3][4];   // per axis: sums of w (far pair, first, second transverse sum, difference)
 #pragma unroll
     for (int a = 0; a < 3; ++a)
@@ -297,22 +298,12 @@ lambda_kernel(Geom g, Mult<double> m, FieldSet<double> lam, const double* e_x, c
     }
     const double x1 = __shfl_down_sync(0xffffffffu, x, 1), x2 = __shfl_down_sync(0xffffffffu, x, 2);
     if (q < 9 && l % 3 == 0)
-        partials[((long long)blockIdx.y * gridDim.x + blockIdx.x) * 9 + q] += x + (x1 + x2);
+        partials[(long long)blockIdx.x * 9 + q] += x + (x1 + x2);
 }
 
 }  // namespace adj64
 
-static dim3 adjoint64_grid(const Geom& g, int& tz) {
-    tz = march64(g, adj64::NL);
-    const long long columns = (seg64::tiles(g) + adj64::NL - 1) / adj64::NL;
-    return dim3((unsigned)columns, (unsigned)((g.nz + tz - 1) / tz));
-}
-
-int adjoint64_blocks(const Geom& g) {
-    int tz;
-    const dim3 d = adjoint64_grid(g, tz);
-    return (int)(d.x * d.y);
-}
+int adjoint64_blocks(const Geom& g) { return (int)march64_grid(g, adj64::NL).blocks; }
 
 void launch_adjoint64(const Geom& g, const Mult<double>& m, FieldSet<double> lam, const double* const E[3],
                       const double* spy, const double* spz, double* partials, cudaStream_t st) {
@@ -320,10 +311,9 @@ void launch_adjoint64(const Geom& g, const Mult<double>& m, FieldSet<double> lam
     const long long pairs = (long long)(g.nx / 2) * g.ny * g.nz, need = (pairs + NT - 1) / NT;
     const unsigned nb = (unsigned)(need < (1 << 20) ? need : (1 << 20));
     launch_pdl(spy ? mu_kernel<true> : mu_kernel<false>, dim3(nb), dim3(NT), 0, st, g, m, lam, spy, spz);
-    int tz;
-    const dim3 grid = adjoint64_grid(g, tz);
-    launch_pdl(spy ? lambda_kernel<true> : lambda_kernel<false>, grid, dim3(NL), 0, st, g, m, lam, E[0],
-               E[1], E[2], spy, spz, partials, tz);
+    const March64 r = march64_grid(g, NL);
+    launch_pdl(spy ? lambda_kernel<true> : lambda_kernel<false>, dim3(r.blocks), dim3(NL), 0, st, g, m, lam,
+               E[0], E[1], E[2], spy, spz, partials, r.tz, r.columns);
 }
 
 }  // namespace fdtd

@@ -191,9 +191,12 @@ __device__ __forceinline__ void dstar_z(const double* Fm, const double* F0, cons
 
 }  // namespace seg64
 
-// Planes a thread of the marching FP64 kernels takes, blocks of `threads` threads: the FP64 pipe is
-// the limit, so the scheduler with the most warps decides, warps x (planes + the first plane's extra
-// differences, a quarter of a plane's work); a single warp takes 1.3 times its share.
-int march64(const Geom& g, int threads);
+// Launch of a marching FP64 kernel in blocks of `threads` threads: `columns` blocks of tiles x chunks
+// of tz planes, the columns fastest, all on one grid axis (a y axis ends at 65535 chunks).
+struct March64 {
+    int tz;
+    unsigned columns, blocks;
+};
+March64 march64_grid(const Geom& g, int threads);
 
 }  // namespace fdtd

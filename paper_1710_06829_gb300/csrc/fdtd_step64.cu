@@ -34,10 +34,12 @@ constexpr int NF = 32;
 template <bool SP>
 __global__ void __launch_bounds__(NF, 3 * NT / NF)
 faraday_kernel(Geom g, Mult<double> m, FieldSet<double> in, FieldSet<double> out,
-               const double* __restrict__ spy, const double* __restrict__ spz, int tz) {
+               const double* __restrict__ spy, const double* __restrict__ spz, int tz,
+               unsigned columns) {
     pdl_wait();
-    const Tile t = tile_of(g, (long long)blockIdx.x * NF + threadIdx.x);
-    const int z0 = blockIdx.y * tz, zend = min(z0 + tz, g.nz);
+    const unsigned chunk = blockIdx.x / columns, column = blockIdx.x - chunk * columns;
+    const Tile t = tile_of(g, (long long)column * NF + threadIdx.x);
+    const int z0 = (int)chunk * tz, zend = min(z0 + tz, g.nz);
     if (t.j < 0) return;
     const double *Ex = in.c[0] + t.o, *Ey = in.c[1] + t.o, *Ez = in.c[2] + t.o;
     const long long Y = g.nxp, y3 = (t.two ? 3 : 2) * Y;
@@ -158,7 +160,10 @@ ampere_kernel(Geom g, Mult<double> m, FieldSet<double> in, FieldSet<double> out,
 
 }  // namespace step64
 
-int march64(const Geom& g, int threads) {
+// Planes a thread takes: the FP64 pipe is the limit, so the scheduler with the most warps decides,
+// warps x (planes + the first plane's extra differences, a quarter of a plane's work); a single warp
+// takes 1.3 times its share.
+static int march64(const Geom& g, int threads) {
     const long long columns = (seg64::tiles(g) + threads - 1) / threads;
     int best = 1;
     double best_cost = -1.0;
@@ -174,15 +179,21 @@ int march64(const Geom& g, int threads) {
     return best;
 }
 
+March64 march64_grid(const Geom& g, int threads) {
+    March64 r;
+    r.tz = march64(g, threads);
+    r.columns = (unsigned)((seg64::tiles(g) + threads - 1) / threads);
+    r.blocks = r.columns * (unsigned)((g.nz + r.tz - 1) / r.tz);
+    return r;
+}
+
 void launch_step64(const Geom& g, const Mult<double>& m, FieldSet<double> in, FieldSet<double> out,
                    const double* spy, const double* spz, const double* jyz, const double* jx_row,
                    double* hist_E[3], int* err, cudaStream_t st) {
     using namespace step64;
-    const int tz = march64(g, NF);
-    const long long tiles = seg64::tiles(g);
-    const dim3 grid((unsigned)((tiles + NF - 1) / NF), (unsigned)((g.nz + tz - 1) / tz));
-    launch_pdl(spy ? faraday_kernel<true> : faraday_kernel<false>, grid, dim3(NF), 0, st, g, m, in, out,
-               spy, spz, tz);
+    const March64 r = march64_grid(g, NF);
+    launch_pdl(spy ? faraday_kernel<true> : faraday_kernel<false>, dim3(r.blocks), dim3(NF), 0, st, g, m, in,
+               out, spy, spz, r.tz, r.columns);
     const long long pairs = (long long)(g.nx / 2) * g.ny * g.nz;
     const unsigned nb = (unsigned)std::min<long long>((pairs + NT - 1) / NT, 1 << 20);
     launch_pdl(spy ? ampere_kernel<true> : ampere_kernel<false>, dim3(nb), dim3(NT), 0, st, g, m, in, out,

@@ -410,3 +410,34 @@ def test_fp32_reverse_step_of_ragged_grids_matches_fp64(shape, dims, kw, monkeyp
     """As above, on grids without whole tiles: down to the smallest that the kernel of four cells a
     thread takes, one to three planes, layers."""
     test_fp32_reverse_step_of_planes_matches_fp64(shape, dims, kw, monkeypatch)
+
+
+def test_fp64_grids_of_more_planes_than_chunks_on_one_grid_axis(monkeypatch):
+    """More z-chunks than a grid's y axis has blocks (chunks of at most 64 planes, 65535 blocks): two
+    recorded steps and the reverse steps against the reference form, whose kernels loop over planes.
+    Tolerances as in test_fp64_reverse_step_matches_the_reference_form."""
+    from paper_1710_06829_gb300 import sim as S
+    shape = (4, 1, 64 * 65535 + 70)
+    if torch.cuda.mem_get_info()[0] < 90 * 2 ** 30:
+        pytest.skip("needs 90 GB of free device memory")
+    gen = torch.Generator(device="cuda").manual_seed(9)
+    f, lam = ([torch.randn(shape[::-1], generator=gen, device="cuda", dtype=torch.float64) for _ in range(6)]
+              for _ in range(2))
+    out = []
+    for flag in ("1", "0"):
+        monkeypatch.setenv("FDTD_FUSED", flag)
+        sm = _sim(shape, "f64")
+        sm.set_state(f)
+        sm.step(2, record=True)
+        state = sm.get_state()
+        sm.set_adjoint(lam)
+        grad = torch.zeros(12, dtype=torch.float64, device="cuda")
+        sm.step_adjoint(2, grad)
+        out.append((state, sm.get_adjoint(), grad))
+        sm.sync()
+        sm.close()
+    for a, b in zip(out[0][0], out[1][0]):
+        assert torch.equal(a, b)
+    for a, b in zip(out[0][1], out[1][1]):
+        assert float((a - b).abs().max()) <= 1e-13 * max(float(c.abs().max()) for c in out[1][1])
+    assert float((out[0][2] - out[1][2]).abs().max()) <= 1e-11 * float(out[1][2].abs().max())
