@@ -1438,25 +1438,28 @@ public:
         if (!ptr) err = cudaMallocAsync((void**)&ptr, doubles * sizeof(double), st);
     }
     // The results (14 doubles at `res` in the scratch, or in the host slot when host_dev was given to
-    // the launch) into `out`: queued before the synchronisation, read after it
+    // the launch) into `out`: queued here, complete after finish()
     cudaError_t copy_out(const double* res, double* out) {
         return host_ ? cudaSuccess : cudaMemcpyAsync(out, res, 14 * sizeof(double), cudaMemcpyDeviceToHost, st_);
     }
-    void read_out(double* out) const {
-        if (host_) memcpy(out, host_, 14 * sizeof(double));
-    }
-    // stream-ordered memory is given back before the call's synchronisation, an area after it
-    void launched() {
-        if (ptr && area_ < 0) cudaFreeAsync(ptr, st_);
-        if (area_ < 0) ptr = nullptr;
-    }
-    ~NormScratch() {
-        launched();
+    // The call's synchronisation: stream-ordered memory is given back before it, an area and its slot
+    // after it and after the results are read.  Also where the call returns with the error e: kernels
+    // that use the area may be queued all the same (an error that an earlier call of the thread left
+    // behind looks like a failed launch).
+    cudaError_t finish(cudaError_t e, double* out) {
+        if (!ptr) return e;
+        if (area_ < 0) cudaFreeAsync(ptr, st_);
+        const cudaError_t s = cudaStreamSynchronize(st_);
+        if (e == cudaSuccess) e = s;
+        if (e == cudaSuccess && host_) memcpy(out, host_, 14 * sizeof(double));
         if (area_ >= 0) {
             std::lock_guard<std::mutex> lock(mutex());
             busy()[dev_][area_] = false;
         }
+        ptr = nullptr;
+        return e;
     }
+    ~NormScratch() { finish(cudaErrorUnknown, nullptr); }   // nothing left to do after finish()
     NormScratch(const NormScratch&) = delete;
     NormScratch& operator=(const NormScratch&) = delete;
     double* ptr = nullptr;
@@ -1530,9 +1533,7 @@ int disp_norm_eval(const fdtd_coeffs* coeffs, double dt, const double dx[3], int
                      scratch.ptr, scratch.host_dev, &res, st);
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) e = scratch.copy_out(res, out);
-    scratch.launched();
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    if (e == cudaSuccess) scratch.read_out(out);
+    e = scratch.finish(e, out);
     if (e != cudaSuccess) {
         set_error("disp_norm_eval: %s", cudaGetErrorString(e));
         return FDTD_ECUDA;
@@ -1574,9 +1575,7 @@ int disp_group_norm_eval(const fdtd_coeffs* coeffs, double dt, const double dx[3
                            scratch.ptr, scratch.host_dev, &res, st);
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) e = scratch.copy_out(res, out);
-    scratch.launched();
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    if (e == cudaSuccess) scratch.read_out(out);
+    e = scratch.finish(e, out);
     if (e != cudaSuccess) {
         set_error("disp_group_norm_eval: %s", cudaGetErrorString(e));
         return FDTD_ECUDA;

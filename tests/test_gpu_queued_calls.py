@@ -82,3 +82,24 @@ def test_steps_probes_and_reverse_steps(shape, dims, dtype, kw):
     for x, y in zip(a, b):
         assert torch.equal(x, y)
     assert float(a[12]) > 0 and float(a[13].abs().max()) > 0
+
+
+def test_norm_call_that_returns_an_error_leaves_no_kernel_behind():
+    """A failed allocation of this thread is still recorded when the norm looks at its launches, so the
+    call may report it; its kernels have ended all the same when it returns, since its scratch is the
+    next call's."""
+    from paper_1710_06829_gb300 import _lib as L
+    from paper_1710_06829_gb300 import sim as S
+    beta, delta = np.zeros((3, 3)), np.zeros(3)
+    args = (beta, delta, 0.5, [1.0, 1.0, 1.0], 3, (256, 256, 256))
+    st = torch.cuda.Stream()
+    ref = S.disp_norm(*args, stream=st)
+    with pytest.raises(L.FdtdError) as ei:   # 12 arrays of 8 TB
+        S.Simulation((10000, 10000, 10000), [1.0, 1.0, 1.0], 0.4, beta, delta, dtype="f64")
+    assert ei.value.status == L.FDTD_ENOMEM
+    try:
+        S.disp_norm(*args, stream=st)
+    except L.FdtdError:
+        pass
+    assert st.query()
+    assert S.disp_norm(*args, stream=st) == ref
