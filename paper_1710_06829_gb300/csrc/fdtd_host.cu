@@ -244,6 +244,8 @@ using namespace fdtd;
         }                                                                               \
     } while (0)
 
+constexpr size_t ERR_BYTES = 256;   // the error flag's part of its allocation
+
 struct fdtd_handle {
     fdtd_grid grid;
     double dx[3];
@@ -272,7 +274,7 @@ struct fdtd_handle {
     cudaEvent_t filled[2];   // ordering events between the handle's stream and the copy stream
     long long step;
     int use_fused;
-    double* dpart;      // diagnostics scratch (block ticket, phase tables, partials)
+    double* dpart;      // diagnostics scratch (block ticket, phase tables, partials), behind err_dev
     std::vector<FusedMaps> hist_maps;   // TMA descriptors of each history snapshot (FP32 adjoint)
     FusedMaps lam_maps;                 // .e[c]: TMA descriptors of lambda_B component c (FP32)
     bool lam_staged = false;            // lam_maps valid: the staged FP32 adjoint E kernel runs
@@ -455,8 +457,12 @@ int fdtd_create(const fdtd_grid* grid, const double dx[3], double dt, const fdtd
     }
     rc = G.dtype == FDTD_F32 ? upload_aux<float>(h) : upload_aux<double>(h);
     if (rc) { fdtd_destroy(h); return rc; }
-    e = cudaMalloc(&h->err_dev, sizeof(int));
-    if (e == cudaSuccess) e = cudaMemsetAsync(h->err_dev, 0, sizeof(int), h->stream);
+    // the error flag and, behind it, the diagnostics' scratch (16 bytes of it start at zero).  Not on
+    // first use: a first step with a probe may be part of a stream capture, which allows neither the
+    // allocation nor a memset that must have run once before the handle's other calls.
+    e = cudaMalloc(&h->err_dev, ERR_BYTES + diag_scratch_bytes(h->g));
+    if (e == cudaSuccess) e = cudaMemsetAsync(h->err_dev, 0, ERR_BYTES + 16, h->stream);
+    h->dpart = (double*)((char*)h->err_dev + ERR_BYTES);
     if (e != cudaSuccess) {
         set_error("cudaMalloc failed: %s", cudaGetErrorString(e));
         fdtd_destroy(h);
@@ -728,18 +734,6 @@ static int ensure_hist(fdtd_handle* h, int snaps) {
     return FDTD_OK;
 }
 
-static int ensure_dpart(fdtd_handle* h) {
-    if (h->dpart) return FDTD_OK;
-    CK(cudaMalloc(&h->dpart, diag_scratch_bytes(h->g)));
-    cudaError_t e = cudaMemsetAsync(h->dpart, 0, 16, h->stream);   // the block ticket
-    if (e != cudaSuccess) {
-        cudaFree(h->dpart);
-        h->dpart = nullptr;
-        CK(e);
-    }
-    return FDTD_OK;
-}
-
 static int ensure_jx(fdtd_handle* h, int n) {
     if (h->jx_cap >= n) return FDTD_OK;
     if (h->jx) { cudaFree(h->jx); h->jx = nullptr; h->jx_cap = 0; }
@@ -838,10 +832,6 @@ static int step_impl(fdtd_handle* h, int n, const fdtd_source* src, const fdtd_p
                               src->q / (h->dx[1] * h->dx[2] * h->dt), h->dx[0], g.nx * h->dx[0],
                               h->step, (T*)h->jx, h->stream);
         CK(cudaGetLastError());
-    }
-    if (probe) {
-        int rc = ensure_dpart(h);
-        if (rc) return rc;
     }
     if (record) {
         int rc = ensure_hist(h, n + 1);
@@ -1093,8 +1083,6 @@ int fdtd_step_adjoint(fdtd_handle* h, int32_t n, const fdtd_probe* probe, double
 int fdtd_diagnostic(fdtd_handle* h, int32_t kind, const double* params, double* out_dev) {
     NvtxRange nvtx_range("fdtd_diagnostic");
     if (!h || !params || !out_dev) { set_error("fdtd_diagnostic: NULL argument"); return FDTD_EINVAL; }
-    int rc = ensure_dpart(h);
-    if (rc) return rc;
     const Geom& g = h->g;
     const bool f32 = h->grid.dtype == FDTD_F32;
     if (kind == FDTD_DIAG_ENERGY) {
@@ -1232,11 +1220,21 @@ static int check_species(const fdtd_handle* h, const fdtd_species* sp, int32_t n
 template <typename T>
 static bool ensure_bmean(fdtd_handle* h) {
     if (h->bmean) return true;
-    if (pic_mean_prepare<T>() &&
-        cudaMalloc(&h->bmean, (size_t)3 * h->g.total * h->esz) == cudaSuccess) return true;
-    h->bmean = nullptr;
-    (void)cudaGetLastError();
-    return false;
+    if (!pic_mean_prepare<T>()) {
+        (void)cudaGetLastError();
+        return false;
+    }
+    // the cycle may be part of a stream capture, or another thread may be capturing: the allocation
+    // (of memory that holds nothing between cycles) must not end it
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    const bool ok = cudaMalloc(&h->bmean, (size_t)3 * h->g.total * h->esz) == cudaSuccess;
+    if (!ok) {
+        h->bmean = nullptr;
+        (void)cudaGetLastError();
+    }
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    return ok;
 }
 
 template <typename T>
@@ -1361,7 +1359,6 @@ void fdtd_destroy(fdtd_handle* h) {
         cudaStreamDestroy(h->xfer);
     }
     if (h->err_dev) cudaFree(h->err_dev);
-    if (h->dpart) cudaFree(h->dpart);
     if (h->plan) fused_plan_destroy(h->plan);
     for (char* p : h->ckpt)
         if (p) cudaFree(p);

@@ -103,3 +103,94 @@ def test_norm_call_that_returns_an_error_leaves_no_kernel_behind():
         pass
     assert st.query()
     assert S.disp_norm(*args, stream=st) == ref
+
+
+def _captured(sm, stream, call):
+    """call() captured as the handle's first of its kind; the graph"""
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=stream):
+        call(sm)
+    return g
+
+
+@pytest.mark.parametrize("shape,dims,dtype,kw", GRIDS)
+def test_first_probe_step_under_stream_capture(shape, dims, dtype, kw):
+    """Two steps with a probe and a plane-wave amplitude, captured as the first calls of a handle and
+    replayed twice, against the same calls made directly."""
+    from paper_1710_06829_gb300 import inputs
+    from paper_1710_06829_gb300 import sim as S
+    beta, delta = inputs.isotropic_theta(-0.05, -0.04, 0.02, 0.01)
+    nx, ny, nz = shape
+    f = [torch.from_numpy(a) for a in inputs.random_fields(shape, 32)]
+    tt = torch.float32 if dtype == "f32" else torch.float64
+    tgt = torch.from_numpy(np.random.default_rng(7).standard_normal((2, nz, ny))).to(tt).repeat(2, 1, 1).cuda()
+    out = []
+    for capture in (False, True):
+        st = torch.cuda.Stream()
+        loss = torch.zeros(1, dtype=torch.float64, device="cuda")
+        amp = torch.zeros(2, dtype=torch.float64, device="cuda")
+        sm = S.Simulation(shape, [1.0, 1.0, 1.0], 0.4, beta, delta, dims=dims, dtype=dtype, stream=st, **kw)
+        sm.set_state(f)
+
+        def call(sm):
+            sm.step(2, probe=S.Probe(0, 1, tgt), loss=loss)
+            sm.plane_wave(4, (0.3, -0.2, 0.1), out=amp)
+        torch.cuda.synchronize()
+        if capture:
+            g = _captured(sm, st, call)
+            with torch.cuda.stream(st):
+                g.replay()
+                g.replay()
+        else:
+            call(sm)
+            call(sm)
+        torch.cuda.synchronize()
+        out.append([*sm.get_state(), loss, amp])
+        sm.sync()
+        sm.close()
+    for a, b in zip(*out):
+        assert torch.equal(a, b)
+
+
+def test_first_cycle_of_many_particles_under_stream_capture():
+    """As above for two PIC cycles with a particle per cell and more (the mean of B formed per cell).
+    The current's additions have no fixed order: about 100 terms of 2e-5 a cell and cycle on fields of
+    0.3, each rounded to 2^-24 of the sum: 4 x 100 x 2^-24 = 2.4e-5 of the largest value at the very
+    most, 1e-5 taken, the roundings having random signs; positions of up to 32 cells by a few 2^-19."""
+    from paper_1710_06829_gb300 import inputs
+    from paper_1710_06829_gb300 import sim as S
+    shape, n = (32, 20, 16), 1 << 20
+    beta, delta = inputs.isotropic_theta(-0.05, -0.04, 0.02, 0.01)
+    gen = torch.Generator(device="cuda").manual_seed(3)
+    ext = torch.tensor(shape, device="cuda", dtype=torch.float32)[:, None]
+    x = torch.rand((3, n), generator=gen, device="cuda") * 0.999 * ext
+    u = torch.randn((3, n), generator=gen, device="cuda")
+    f = [torch.from_numpy(0.1 * a) for a in inputs.random_fields(shape, 33)]
+    out = []
+    for capture in (False, True):
+        st = torch.cuda.Stream()
+        sm = S.Simulation(shape, [1.0, 1.0, 1.0], 0.4, beta, delta, dtype="f32", stream=st)
+        sm.set_state(f)
+        sp = S.Species(x.clone(), u.clone(), 2e-5, -1.0)
+
+        def call(sm):
+            sm.pic_step(2, [sp])
+        torch.cuda.synchronize()
+        if capture:
+            g = _captured(sm, st, call)
+            with torch.cuda.stream(st):
+                g.replay()
+                g.replay()
+        else:
+            call(sm)
+            call(sm)
+        torch.cuda.synchronize()
+        out.append((sm.get_state(), sp))
+        sm.sync()
+        sm.close()
+    big = max(float(a.abs().max()) for a in out[0][0])
+    for a, b in zip(out[0][0], out[1][0]):
+        assert float((a - b).abs().max()) <= 1e-5 * big
+    d = (out[0][1].x - out[1][1].x).abs()
+    assert float(torch.minimum(d, ext - d).max()) <= 1e-4
+    assert float((out[0][1].u - out[1][1].u).abs().max()) <= 1e-4
