@@ -150,8 +150,13 @@ struct Vec<double> {
 // (denormals included), since the float's exponent field is placed in the double's as it is.  The
 // conversion instruction runs on the FP64 pipe (two lanes an SM), where it would cost as much as
 // a multiply-add.  `top` collects the magnitudes' bits: 0x7f800000 or more tells that an infinity
-// or a NaN was among them, which this form does not carry over.
+// or a NaN was among them, which this form does not carry over; and where the largest is below 2^-120,
+// products with a phase fall below the normal doubles and lose digits (above it at most 2^-59 of the
+// largest value).  Such values are converted instead.
 constexpr double WIDEN_BACK = 0x1p896;
+__device__ __forceinline__ bool widens(unsigned top) {
+    return top == 0 || (top >= 0x03800000u && top < 0x7f800000u);
+}
 __device__ __forceinline__ void widen(const float* p, double* v, unsigned& top) {
     const uint4 a = *reinterpret_cast<const uint4*>(p);
     const unsigned b[4] = {a.x, a.y, a.z, a.w};
@@ -220,7 +225,7 @@ planewave_kernel(Geom g, const T* F, const double2* tab, double* part,
         const T* p = F + pidx(g, it.i, it.j0, it.k);
         const double2* ey = tab + g.nx + it.j0;
         double re[V], im[V];
-        bool finite = true;
+        bool plain = true;   // the row sums hold
         const int rows = it.j1 - it.j0;
         auto rows_sum = [&](auto&& load) {
 #pragma unroll
@@ -242,17 +247,17 @@ planewave_kernel(Geom g, const T* F, const double2* tab, double* part,
             rows_sum([&](const float* q, double* v) { widen(q, v, top); });
 #pragma unroll
             for (int u = 0; u < V; ++u) { re[u] *= WIDEN_BACK; im[u] *= WIDEN_BACK; }
-            finite = top < 0x7f800000u;
+            plain = widens(top);
         } else {
             rows_sum([&](const T* q, double* v) { Vec<T>::load(q, v); });
 #pragma unroll
-            for (int u = 0; u < V; ++u) finite = finite && isfinite(re[u]) && isfinite(im[u]);
+            for (int u = 0; u < V; ++u) plain = plain && isfinite(re[u]) && isfinite(im[u]);
         }
         const double2 ez = tab[g.nx + g.ny + it.k];
         auto times = [](double2 a, double2 b) {
             return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
         };
-        if (finite) {
+        if (plain) {
             double2 c = make_double2(0.0, 0.0);
 #pragma unroll
             for (int u = 0; u < V; ++u) {
@@ -263,7 +268,7 @@ planewave_kernel(Geom g, const T* F, const double2* tab, double* part,
             c = times(c, ez);
             acc[0] += c.x;
             acc[1] -= c.y;
-        } else {   // infinities reach the sums as value x phase, cell by cell
+        } else {   // cell by cell: infinities reach the sums as value x phase
             for (int j = 0; j < rows; ++j)
                 for (int u = 0; u < V; ++u) {
                     const double2 e = times(times(tab[it.i + u], ey[j]), ez);

@@ -80,6 +80,27 @@ def test_plane_wave_of_denormals_and_non_finite_values():
     sm.close()
 
 
+@pytest.mark.parametrize("scale", [1.4e-45, 1e-42, 1e-38, 1e-36, 1e-30])
+def test_plane_wave_of_tiny_fields(scale):
+    """Fields of a few denormal steps up to small normal ones, with a phase, one column group of ordinary
+    size among those of the second plane: tolerance of test_projections_match_direct_sums."""
+    from paper_1710_06829_gb300 import inputs
+    shape = (24, 35, 2)
+    f = np.random.default_rng(12).integers(-40, 41, size=shape[::-1]).astype(np.float64) * scale
+    f[1, 20, 4:8] *= 1e6
+    f = f.astype(np.float32).astype(np.float64)
+    sm = _sim(shape)
+    sm.set_state([torch.from_numpy(f)] + [None] * 5)
+    for k in ((0.3, -0.7, 1.1), (2.9, 0.01, -3.0)):
+        x, y, z = inputs.positions(shape, 0, [1.0, 1.0, 1.0])
+        ph = np.exp(-1j * (k[0] * x + k[1] * y + k[2] * z))
+        for part in (f, np.where(np.arange(2)[:, None, None] == 0, f, 0.0)):   # both planes, one of them
+            sm.set_state([torch.from_numpy(part)] + [None] * 5)
+            got = sm.plane_wave(0, k).cpu().numpy()
+            assert abs(got[0] + 1j * got[1] - np.sum(part * ph)) <= 1e-13 * np.sum(np.abs(part))
+    sm.close()
+
+
 @pytest.mark.parametrize("offset", [0, 1])
 @pytest.mark.parametrize("dtype", ["f32", "f64"])
 @pytest.mark.parametrize("shape,dims", [((4, 1, 1), 1), ((8, 3, 1), 2), ((260, 5, 7), 3), ((68, 130, 9), 3)])
