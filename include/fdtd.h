@@ -273,8 +273,8 @@ int fdtd_selftest_wait_expiry(fdtd_handle* h, int32_t tries);
  * s+1, then step n+2 of slab s, so that the intermediate state (E^{n+1}, B^{n+1/2}) is read
  * back from L2 while it is still resident, and the intermediate planes no later launch needs
  * are dropped from L2 without being written to DRAM.  slab_planes (>= 3; 0 = 32) sets the slab
- * length.  Applies to FP32 grids on the fused path (nx >= 8, ny >= 4, nz >= 4) with at least
- * two slabs, and to fdtd_step calls without a source, probe or history; other calls, and an
+ * length.  Applies to FP32 grids on the fused path (nx >= 8, ny >= 4, nz >= 4, not batched) with at
+ * least two slabs, and to fdtd_step calls without a source, probe or history; other calls, and an
  * odd last step, run one launch per step.  T = 1 (the default) restores one launch per step.
  * Returns FDTD_EINVAL for other T or slab_planes in 1 .. 2. */
 int fdtd_set_temporal_blocking(fdtd_handle* h, int32_t T, int32_t slab_planes);

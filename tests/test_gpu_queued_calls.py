@@ -194,3 +194,27 @@ def test_first_cycle_of_many_particles_under_stream_capture():
     d = (out[0][1].x - out[1][1].x).abs()
     assert float(torch.minimum(d, ext - d).max()) <= 1e-4
     assert float((out[0][1].u - out[1][1].u).abs().max()) <= 1e-4
+
+
+@pytest.mark.parametrize("shape", [(64, 16, 8), (60, 14, 9)])
+def test_temporal_blocking_keeps_the_problems_of_a_batch_apart(shape):
+    """Pairs of steps on a batch: the bits of single steps, and an infinity in one problem stays there (a
+    zero multiplier of a z difference would carry it to the neighbouring ones as NaN)."""
+    from paper_1710_06829_gb300 import inputs
+    from paper_1710_06829_gb300 import sim as S
+    beta, delta = inputs.isotropic_theta(-0.05, -0.04, 0.02, 0.01)
+    out = []
+    for T, bad in ((1, False), (2, False), (2, True)):
+        f = [torch.from_numpy(a) for a in inputs.random_fields(shape, 34)]
+        if bad:
+            f[0][3, 5, 7] = float("inf")
+        sm = S.Simulation(shape, [1.0, 1.0, 1.0], 0.4, beta, delta, dims=2, dtype="f32", batched=True)
+        sm.set_temporal_blocking(T, 3)
+        sm.set_state(f)
+        sm.step(5)
+        out.append(sm.get_state())
+        sm.close()
+    for a, b, c in zip(*out):
+        assert torch.equal(a, b)
+        c = torch.cat([c[:3], c[4:]])
+        assert torch.equal(torch.cat([a[:3], a[4:]]), c)
