@@ -40,6 +40,7 @@ void launch_step2d32(const Geom& g, const Mult<float>& m, FieldSet<float> in, Fi
                      const float* spy, const float* spz, const float* jyz, const float* jx_row,
                      float* hist_E[3], int* err, cudaStream_t st);
 
+bool step2d64_prepare();
 void launch_step2d64(const Geom& g, const Mult<double>& m, FieldSet<double> in, FieldSet<double> out,
                      const double* spy, const double* spz, const double* jyz, const double* jx_row,
                      double* hist_E[3], int* err, cudaStream_t st);
@@ -100,7 +101,7 @@ FusedPlan* fused_plan_create(const Geom& g, bool flat, T* const set0[6], T* cons
         }
         ok = fused32_prepare();
     } else {
-        ok = true;
+        ok = !flat || step2d64_prepare();
     }
     if (!ok) {
         delete p;

@@ -28,6 +28,10 @@ struct Cfg {
     static constexpr int YW = TX + 3, YH = TY + 1;   // y differences: x0-2 .. x0+TX, y0-1 .. y0+TY-1
     static constexpr int BW = TX + 1, BH = TY + 1;   // B: x0-1 .. x0+TX-1, y0-1 .. y0+TY-1
     static constexpr int NB = (BW * BH + NT - 1) / NT;
+    static constexpr int EN = EW * EH, XN = XW * XH, YN = YW * YH, BN = BW * BH;
+    // dynamic shared memory: 15160 bytes of the small tile, 50296 of the large one (static shared
+    // memory ends at 48 KB)
+    static constexpr size_t SMEM = (3 * EN + 2 * XN + 2 * YN + 3 * BN) * sizeof(double);
 };
 
 __device__ __forceinline__ bool nonfinite(double v) {
@@ -44,9 +48,12 @@ step2d64_kernel(Geom g, Mult<double> m, FieldSet<double> in, FieldSet<double> ou
                 int* __restrict__ err) {
     using C = Cfg<TX, TY>;
     constexpr int EW = C::EW, XW = C::XW, YW = C::YW, BW = C::BW, NT = C::NT;
-    __shared__ __align__(16) double sE[3][C::EH * EW];
-    __shared__ double sX[2][C::XH * XW], sY[2][C::YH * YW];   // d_x of E_y, E_z; d_y of E_x, E_z
-    __shared__ double sB[3][C::BH * BW];
+    extern __shared__ __align__(16) double smem64[];
+    double (*sE)[C::EN] = reinterpret_cast<double (*)[C::EN]>(smem64);
+    double (*sX)[C::XN] = reinterpret_cast<double (*)[C::XN]>(smem64 + 3 * C::EN);   // d_x of E_y, E_z
+    double (*sY)[C::YN] = reinterpret_cast<double (*)[C::YN]>(sX + 2);               // d_y of E_x, E_z
+    double (*sB)[C::BN] = reinterpret_cast<double (*)[C::BN]>(sY + 2);
+    static_assert(C::EW % 2 == 0, "rows of the E box start on 16 bytes");
     pdl_wait();
     const int ntx = (g.nx + TX - 1) / TX, nty = (g.ny + TY - 1) / TY;
     int w = blockIdx.x;
@@ -160,6 +167,16 @@ step2d64_kernel(Geom g, Mult<double> m, FieldSet<double> in, FieldSet<double> ou
 
 }  // namespace flat64
 
+// before the first launch: room for the large tile's shared memory
+bool step2d64_prepare() {
+    using namespace flat64;
+    bool ok = true;
+    for (auto kern : {step2d64_kernel<32, 16, false>, step2d64_kernel<32, 16, true>})
+        ok = ok && cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                        (int)Cfg<32, 16>::SMEM) == cudaSuccess;
+    return ok;
+}
+
 void launch_step2d64(const Geom& g, const Mult<double>& m, FieldSet<double> in, FieldSet<double> out,
                      const double* spy, const double* spz, const double* jyz, const double* jx_row,
                      double* hist_E[3], int* err, cudaStream_t st) {
@@ -169,7 +186,7 @@ void launch_step2d64(const Geom& g, const Mult<double>& m, FieldSet<double> in, 
         const long long tiles = (long long)((g.nx + TX - 1) / TX) * ((g.ny + TY - 1) / TY) * g.nz;
         const bool zc = m.cB[0][2] != 0.0 || m.cB[1][2] != 0.0;
         launch_pdl(zc ? step2d64_kernel<TX, TY, true> : step2d64_kernel<TX, TY, false>,
-                   dim3((unsigned)tiles), dim3(Cfg<TX, TY>::NT), 0, st, g, m, in, out, spy, spz, jyz,
+                   dim3((unsigned)tiles), dim3(Cfg<TX, TY>::NT), Cfg<TX, TY>::SMEM, st, g, m, in, out, spy, spz, jyz,
                    jx_row, hist_E[0], hist_E[1], hist_E[2], err);
     };
     // Small tiles reach more SMs and schedulers, large ones form fewer halo values (us, 16 x 8 / 32 x 16:

@@ -263,6 +263,16 @@ def test_planes_step_bitwise_like_the_reference_form(nx, ny, nz, batched, dtype,
         assert torch.equal(a, b)
 
 
+@pytest.mark.parametrize("shape,batched", [((1004, 701, 1), False), ((68, 33, 320), True),
+                                           ((1004, 701, 1), None), ((512, 1368, 1), False)])
+def test_large_fp64_planes_step_bitwise_like_the_reference_form(shape, batched, monkeypatch):
+    """As above from 700000 cells on, where the FP64 kernel takes its large tile: ragged in both directions,
+    a batch with layers, a 3D problem one plane thick, whole tiles."""
+    kw = dict(batched=True, absorb_cells=2, absorb_sigma=0.3) if batched else {}
+    for a, b in zip(*_step_pair(shape, "f64", monkeypatch, dims=3 if batched is None else 2, **kw)):
+        assert torch.equal(a, b)
+
+
 # one warp, a ragged warp, several blocks; particles of one cell moving across no, one or three faces
 # and both ways along an axis (momenta along the cell's diagonal, or random), grids of a few cells, the
 # per-cell mean of B (at least 2^20 particles and one per cell)
