@@ -218,3 +218,26 @@ def test_temporal_blocking_keeps_the_problems_of_a_batch_apart(shape):
         assert torch.equal(a, b)
         c = torch.cat([c[:3], c[4:]])
         assert torch.equal(torch.cat([a[:3], a[4:]]), c)
+
+
+@pytest.mark.parametrize("shape,slab,sponge", [((60, 12, 20), 4, False), ((132, 15, 33), 5, True),
+                                               ((8, 4, 9), 3, False), ((68, 9, 70), 0, False)])
+def test_temporal_blocking_on_ragged_grids(shape, slab, sponge):
+    """Pairs of steps give the bits of single steps on grids without whole tiles too."""
+    from paper_1710_06829_gb300 import inputs
+    from paper_1710_06829_gb300 import sim as S
+    beta, delta = inputs.isotropic_theta(-0.05, -0.04, 0.02, 0.01)
+    f = [torch.from_numpy(a) for a in inputs.random_fields(shape, 35)]
+    kw = dict(absorb_cells=2, absorb_sigma=0.2) if sponge else {}
+    out = []
+    for T in (1, 2):
+        sm = S.Simulation(shape, [1.0, 1.0, 1.0], 0.4, beta, delta, dtype="f32", **kw)
+        sm.set_temporal_blocking(T, slab)
+        sm.set_state(f)
+        sm.step(5)
+        sm.step(2)
+        sm.sync()
+        out.append(sm.get_state())
+        sm.close()
+    for a, b in zip(*out):
+        assert torch.equal(a, b)
