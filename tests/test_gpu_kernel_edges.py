@@ -472,3 +472,54 @@ def test_fp64_grids_of_more_planes_than_chunks_on_one_grid_axis(monkeypatch):
     for a, b in zip(out[0][1], out[1][1]):
         assert float((a - b).abs().max()) <= 1e-13 * max(float(c.abs().max()) for c in out[1][1])
     assert float((out[0][2] - out[1][2]).abs().max()) <= 1e-11 * float(out[1][2].abs().max())
+
+
+@pytest.mark.parametrize("sponge", [False, True])
+@pytest.mark.parametrize("shape,per,extra", [((32, 32, 32), 32, 0), ((32, 16, 32), 64, 77)])
+def test_push_of_many_particles_in_cell_order_matches_the_oracle(shape, per, extra, sponge):
+    """FP32, at least 2^20 charged particles, whole warps in one cell: their currents are summed through
+    the shared rows of all 24 warps of the large block.  By cell, particles at rest, moving along x,
+    along the diagonal (over one to three faces, some and not others) and every way; extra particles
+    shift the last warps off the cells.  Against the FP64 oracle on the same FP32 inputs: positions of up
+    to 32 cells are rounded to 2^-20 of a cell where a particle moves by 0.4, so a face's sum is good to
+    about 5e-6 of its terms, fields included; 5e-5 of the largest value taken."""
+    from oracle import dispersion as D
+    from oracle import fdtd as F
+    from oracle import pic as P
+    from paper_1710_06829_gb300 import inputs
+    from paper_1710_06829_gb300 import sim as S
+    nx, ny, nz = shape
+    beta, delta = inputs.isotropic_theta(-0.05, -0.04, 0.02, 0.01)
+    dx = [1.0, 1.0, 1.0]
+    dt = 0.95 * D.dt_max(beta, delta, dx, 3)
+    rng = np.random.default_rng(per)
+    cells = nx * ny * nz
+    c = np.repeat(np.arange(cells), per)
+    n = c.size
+    origin = np.array([c % nx, c // nx % ny, c // (nx * ny)], dtype=np.float64)
+    x = (origin + rng.uniform(0.0, 0.999, (3, n))).astype(np.float32)
+    way = rng.choice([-1.0, 1.0], (3, cells))[:, c]
+    kinds = np.stack([np.zeros((3, n)), way * np.array([[4.0], [0.0], [0.0]]), 3.0 * way,
+                      3.0 * rng.standard_normal((3, n))])
+    u = np.take_along_axis(kinds, (c % 4)[None, None, :], axis=0)[0].astype(np.float32)
+    if extra:
+        x = np.concatenate([x[:, :1000], rng.uniform(0.0, 0.999, (3, extra)).astype(np.float32), x[:, 1000:]], axis=1)
+        u = np.concatenate([u[:, :1000], np.zeros((3, extra), np.float32), u[:, 1000:]], axis=1)
+    f = [(0.01 * a).astype(np.float32) for a in inputs.random_fields(shape, 8)]
+    kw = dict(absorb_cells=4, absorb_sigma=0.3) if sponge else {}
+    q = 1.0 / per
+    sm = S.Simulation(shape, dx, dt, beta, delta, dtype="f32", **kw)
+    sm.set_state([torch.from_numpy(a) for a in f])
+    sp = S.Species(torch.from_numpy(x.copy()).cuda(), torch.from_numpy(u.copy()).cuda(), q, -1.0)
+    sm.pic_step(1, [sp])
+    sm.sync()
+    got = [t.double().cpu().numpy() for t in sm.get_state()]
+    sm.close()
+    f64 = [a.astype(np.float64) for a in f]
+    st, pt = F.State(f64[:3], f64[3:]), P.Particles(x.astype(np.float64), u.astype(np.float64), q, -1.0)
+    fac = F.sponge_factor((nz, ny, nx), 4, 0.3) if sponge else None
+    st = P.pic_step(st, [pt], F.Coeffs(beta, delta, dx, dt), fac)
+    big = max(float(np.max(np.abs(v))) for v in st.E)
+    assert big > 0.1   # the currents, not the fields of 0.01
+    for a, b in zip(got, st.E + st.B):
+        assert np.max(np.abs(a - b)) <= 5e-5 * big
