@@ -107,7 +107,11 @@ __device__ __forceinline__ void root_both(double a, double& s, double& rs) {
     rs = fma(e * r, t, r);
 }
 
-// a normal positive double's value in single precision (truncated), by integer shifts
+// a positive double between 2^-126 and 2^127, and its value in single precision (truncated), by integer
+// shifts
+__device__ __forceinline__ bool narrows(double x) {
+    return (unsigned)__double2hiint(x) - 0x38100000u < 0x0fd00000u;
+}
 __device__ __forceinline__ float narrow(double x) {
     return __uint_as_float(((unsigned)(__double2hiint(x) - 0x38000000) << 3) |
                            ((unsigned)__double2loint(x) >> 29));
@@ -116,9 +120,11 @@ __device__ __forceinline__ float narrow(double x) {
 // the cone's weight at (kx, ky, kz): single precision decides away from the cone's surface (its
 // error is below 1e-6 of either side), the FP64 expression next to it
 __device__ __forceinline__ bool in_cone(double kx, double ky, double kz, double cos_half) {
-    const float x = narrow(kx), y = ky > 0.0 ? narrow(ky) : 0.0f, z = kz > 0.0 ? narrow(kz) : 0.0f;
-    const float n = sqrtf(x * x + y * y + z * z), c = n * (float)cos_half;
-    if (n > 1e-15f && n < 1e15f && fabsf(x - c) > 1e-5f * n) return x > c;
+    if (narrows(kx) && (ky == 0.0 || narrows(ky)) && (kz == 0.0 || narrows(kz))) {
+        const float x = narrow(kx), y = ky > 0.0 ? narrow(ky) : 0.0f, z = kz > 0.0 ? narrow(kz) : 0.0f;
+        const float n = sqrtf(x * x + y * y + z * z), c = n * (float)cos_half;
+        if (n > 1e-15f && n < 1e15f && fabsf(x - c) > 1e-5f * n) return x > c;
+    }
     return kx >= sqrt(kx * kx + ky * ky + kz * kz) * cos_half;
 }
 
@@ -210,8 +216,8 @@ norm_kernel(NormParams p, const double2* __restrict__ tab, const Angle* __restri
             double x = p.dt * sq;
             const double q = fma(-x, x, 1.0);
             double c, rc, th;
-            // both positive, S between 2^-126 and 2^127, x and q between 2^-63 and 1: integer comparisons
-            if ((unsigned)__double2hiint(S) - 0x38100000u < 0x0fd00000u &&
+            // S between 2^-126 and 2^127, x and q positive, between 2^-63 and 1: integer comparisons
+            if (narrows(S) &&
                 (unsigned)__double2hiint(x) - 0x3c000000u < 0x04000000u &&
                 (unsigned)__double2hiint(q) - 0x3c000000u < 0x04000000u) {
                 root_both(q, c, rc);

@@ -166,6 +166,21 @@ def test_norm_segments_and_weights_match_oracle(dims, N, courant, weight, par):
     assert np.all(np.abs(got - ref) <= 1e-11 * np.abs(ref) + 1e-13 * max(1.0, abs(rf)))
 
 
+@pytest.mark.parametrize("weight,par", [(0, 0.0), (1, math.radians(30))])
+@pytest.mark.parametrize("e", [-250, -140, 140, 250])
+def test_norm_of_wave_numbers_outside_the_float_range(e, weight, par):
+    """Spacings of 1 and 2^e: the wave numbers of one axis lie outside single precision's range, in which
+    the cone's test is made where it can be.  Yee's scheme; tolerance as above."""
+    from oracle import dispersion as D
+    from paper_1710_06829_gb300 import sim as S
+    beta, delta, dx, N = np.zeros((3, 3)), np.zeros(3), [1.0, 2.0 ** e, 1.0], (40, 33, 1)
+    dt = 0.9 * D.dt_max(beta, delta, dx, 2)
+    f, gb, gd, gdt = S.disp_norm(beta, delta, dt, dx, 2, N, weight, par)
+    rf, rgb, rgd, rgdt = D.norm_and_grad(beta, delta, dt, dx, N, 2, (D.WEIGHT_UNIFORM, D.WEIGHT_CONE_X)[weight], par)
+    got, ref = np.r_[f, np.ravel(gb), gd, gdt], np.r_[rf, np.ravel(rgb), rgd, rgdt]
+    assert np.all(np.abs(got - ref) <= 1e-11 * np.abs(ref) + 1e-13 * max(1.0, abs(rf)))
+
+
 def test_norm_from_several_threads_and_streams():
     """More concurrent evaluations than scratch areas: every one returns its own value."""
     import threading
