@@ -55,53 +55,42 @@ bool fused_supported(const Geom& g, bool flat) {
     return true;   // fdtd_step2d64.cu and fdtd_step64.cu take every size
 }
 
-template <typename T>
-static bool encode(CUtensorMap* map, const Geom& g, T* base, int bw, int bh) {
+// a bw x bh box (FP32) of one padded array
+bool encode_box_f32(CUtensorMap* map, const Geom& g, float* base, int bw, int bh) {
     EncodeTiledFn fn = encode_fn();
     if (!fn) return false;
     const cuuint64_t dims[3] = {(cuuint64_t)g.nxp, (cuuint64_t)g.nyp, (cuuint64_t)g.nz};
-    const cuuint64_t strides[2] = {(cuuint64_t)g.nxp * sizeof(T), (cuuint64_t)g.plane * sizeof(T)};
+    const cuuint64_t strides[2] = {(cuuint64_t)g.nxp * 4, (cuuint64_t)g.plane * 4};
     const cuuint32_t box[3] = {(cuuint32_t)bw, (cuuint32_t)bh, 1};
     const cuuint32_t estr[3] = {1, 1, 1};
-    const CUtensorMapDataType dt =
-        sizeof(T) == 4 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_FLOAT64;
-    return fn(map, dt, 3, (void*)base, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-              CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+    return fn(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, base, dims, strides, box, estr,
+              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 // E^n box (x0-4 .., y0-2 .. of a 64 x 8 tile: 72 x 12, FP32) of one padded array, as the adjoint
 // kernels read it
 bool encode_ebox_f32(CUtensorMap* map, const Geom& g, float* base) {
-    return encode<float>(map, g, base, 72, 12);
-}
-
-// a bw x bh box (FP32) of one padded array
-bool encode_box_f32(CUtensorMap* map, const Geom& g, float* base, int bw, int bh) {
-    return encode<float>(map, g, base, bw, bh);
+    return encode_box_f32(map, g, base, 72, 12);
 }
 
 template <typename T>
 FusedPlan* fused_plan_create(const Geom& g, bool flat, T* const set0[6], T* const set1[6]) {
     if (!fused_supported<T>(g, flat)) return nullptr;
     FusedPlan* p = new FusedPlan();
-    p->dtype = sizeof(T) == 4 ? FDTD_F32 : FDTD_F64;
     p->flat = flat;
-    bool ok;
+    bool ok = true;
     if constexpr (std::is_same<T, float>::value) {
         for (int s = 0; s < 2; ++s) {
             T* const* set = s == 0 ? set0 : set1;
+            // E boxes x0-4 .., y0-2 ..; B boxes x0-4 .., y0-1 .. (68 x 9)
             for (int c = 0; c < 3; ++c)
-                // E boxes x0-4 .., y0-2 ..; B boxes x0-4 .., y0-1 .. (68 x 9)
-                if (!encode<T>(&p->maps[s].e[c], g, set[c], fused32_ebox_w(), 12) ||
-                    !encode<T>(&p->maps[s].b[c], g, set[3 + c], 68, 9)) {
-                    delete p;
-                    return nullptr;
-                }
+                ok = ok && encode_box_f32(&p->maps[s].e[c], g, set[c], fused32_ebox_w(), 12) &&
+                     encode_box_f32(&p->maps[s].b[c], g, set[3 + c], 68, 9);
         }
-        ok = fused32_prepare();
-    } else {
-        ok = !flat || step2d64_prepare();
+        ok = ok && fused32_prepare();
+    } else if (flat) {
+        ok = step2d64_prepare();
     }
     if (!ok) {
         delete p;

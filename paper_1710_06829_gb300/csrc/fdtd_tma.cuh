@@ -14,7 +14,6 @@ struct FusedMaps {
 };
 
 struct FusedPlan {
-    int dtype;
     bool flat;           // the planes do not couple along z (nz = 1, or a batch of 2D problems)
     FusedMaps maps[2];   // indexed by input set
 };
