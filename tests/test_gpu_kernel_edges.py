@@ -538,3 +538,29 @@ def test_push_of_many_particles_in_cell_order_matches_the_oracle(shape, per, ext
     assert big > 0.1   # the currents, not the fields of 0.01
     for a, b in zip(got, st.E + st.B):
         assert np.max(np.abs(a - b)) <= 5e-5 * big
+
+
+@pytest.mark.parametrize("shape,dims,kw", [
+    ((64, 8, 1), 2, {}), ((64, 16, 1), 3, {}), ((192, 8, 17), 2, dict(batched=True)),
+    ((128, 24, 70), 2, dict(batched=True, absorb_cells=3, absorb_sigma=0.3))])
+def test_fp32_reverse_step_of_planes_is_bitwise_that_of_the_3d_kernels(shape, dims, kw, monkeypatch):
+    """lambda of the 2D kernel against the two-kernel 3D form, which forms every value in the same order."""
+    from paper_1710_06829_gb300 import sim as S
+    f = [torch.from_numpy(a) for a in _random_state(shape, "f32", 16)]
+    lam = [torch.from_numpy(a) for a in _random_state(shape, "f32", 17)]
+    nx, ny, nz = shape
+    tgt = torch.from_numpy(np.random.default_rng(5).standard_normal((3, nz, ny)).astype(np.float32)).cuda()
+    out = []
+    for flag in ("0", "1"):
+        monkeypatch.setenv("FDTD_ADJOINT_SPLIT", flag)
+        sm = _sim(shape, "f32", dims=dims, **kw)
+        sm.set_state(f)
+        sm.step(3, record=True)
+        sm.set_adjoint(lam)
+        grad = torch.zeros(12, dtype=torch.float64, device="cuda")
+        sm.step_adjoint(3, grad, probe=S.Probe(1, nx - 1, tgt))
+        out.append((sm.get_adjoint(), grad))
+        sm.sync()
+        sm.close()
+    for a, b in zip(out[0][0], out[1][0]):
+        assert torch.equal(a, b)
