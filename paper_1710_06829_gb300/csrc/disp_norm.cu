@@ -30,6 +30,8 @@
 // A thread takes one row segment at a time, neighbouring threads neighbouring k_y; a block's sums
 // are taken once, and the block that arrives last adds the blocks' partials in a fixed order
 // (deterministic result).
+#include <math_constants.h>
+
 #include <cmath>
 
 #include "fdtd_internal.cuh"
@@ -118,11 +120,16 @@ __device__ __forceinline__ float narrow(double x) {
 }
 
 // the cone's weight at (kx, ky, kz): single precision decides away from the cone's surface (its
-// error is below 1e-6 of either side), the FP64 expression next to it
-__device__ __forceinline__ bool in_cone(double kx, double ky, double kz, double cos_half) {
-    if (narrows(kx) && (ky == 0.0 || narrows(ky)) && (kz == 0.0 || narrows(kz))) {
-        const float x = narrow(kx), y = ky > 0.0 ? narrow(ky) : 0.0f, z = kz > 0.0 ? narrow(kz) : 0.0f;
-        const float n = sqrtf(x * x + y * y + z * z), c = n * (float)cos_half;
+// error is below 1e-6 of either side), the FP64 expression next to it and outside the float range.
+// t2: ky^2 + kz^2 of the row in single precision, NaN where that cannot be formed
+__device__ __forceinline__ float cone_row(double ky, double kz) {
+    if ((ky != 0.0 && !narrows(ky)) || (kz != 0.0 && !narrows(kz))) return CUDART_NAN_F;
+    const float y = ky > 0.0 ? narrow(ky) : 0.0f, z = kz > 0.0 ? narrow(kz) : 0.0f;
+    return y * y + z * z;
+}
+__device__ __forceinline__ bool in_cone(double kx, double ky, double kz, float t2, double cos_half) {
+    if (narrows(kx)) {
+        const float x = narrow(kx), n = sqrtf(x * x + t2), c = n * (float)cos_half;
         if (n > 1e-15f && n < 1e15f && fabsf(x - c) > 1e-5f * n) return x > c;
     }
     return kx >= sqrt(kx * kx + ky * ky + kz * kz) * cos_half;
@@ -185,12 +192,13 @@ norm_kernel(NormParams p, const double2* __restrict__ tab, const Angle* __restri
         double w = 1.0;
         if (p.weight == FDTD_W_CONE_X) {
             // along the row the weight is 0 up to an index and 1 from it on
-            if (!in_cone(tab[m1 - 1].x, y.x, z.x, p.wparam)) continue;
-            if (!in_cone(tab[m0].x, y.x, z.x, p.wparam)) {
+            const float t2 = cone_row(y.x, z.x);
+            if (!in_cone(tab[m1 - 1].x, y.x, z.x, t2, p.wparam)) continue;
+            if (!in_cone(tab[m0].x, y.x, z.x, t2, p.wparam)) {
                 int lo = m0, hi = m1 - 1;   // outside at lo, inside at hi
                 while (hi - lo > 1) {
                     const int mid = (lo + hi) >> 1;
-                    if (in_cone(tab[mid].x, y.x, z.x, p.wparam)) hi = mid;
+                    if (in_cone(tab[mid].x, y.x, z.x, t2, p.wparam)) hi = mid;
                     else lo = mid;
                 }
                 m0 = hi;

@@ -14,8 +14,8 @@
 //
 // The z differences are the plane's own (nz = 1) or have zero multipliers (batch): D*_z and the
 // third gradient term of D*_x and D*_y (T_beta_az, exactly zero or not asked for) drop out.  Every
-// sum is taken over the same cells in the same order as there (the chunk's planes are one
-// compensated FP32 sum a thread and axis), so lambda and the gradient are bitwise those of that kernel.
+// value is formed and every sum taken over the same cells in the same order as there (the chunk's
+// planes are one compensated FP32 sum a thread and axis); lambda is bitwise that of the 3D kernels.
 //
 // Bound: HBM for a large batch (60 B a cell), launch and latency for a small one.  Us a step, the 3D
 // kernel and this one: 512 x 512 x 32 148 / 97 (503 MB: 0.76 of the copy rate), 512 x 512 x 8 50 / 29,

@@ -648,7 +648,7 @@ int adjoint32f_blocks(const Geom& g) {
 // maps.e[c]: 72 x 12 boxes of lambda_E component c of the input set `lam`, maps.b[c]: 72 x 11
 // boxes of its lambda_B component c; E: the forward
 // E^n of the step (padded arrays); the result goes to `out` (the other set).  Planes that do not
-// couple along z (flat) take the kernel without halo planes (fdtd_adjoint2d.cu), same results
+// couple along z (flat) take the kernel without halo planes (fdtd_adjoint2d.cu)
 void launch_adjoint32_fused(const FusedMaps& maps, const Geom& g, const Mult<float>& m,
                             FieldSet<float> lam, FieldSet<float> out, const float* const E[3],
                             const float* spy, const float* spz, double* partials, bool flat,

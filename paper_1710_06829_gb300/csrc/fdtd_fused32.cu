@@ -8,11 +8,11 @@
 // A CTA owns a 64 x 8 (x, y) tile and a chunk of tz planes (a launch parameter) and marches
 // through it; the last tiles of a ragged grid reach past its cells and drop what they form there.
 // E^n planes arrive by TMA (cp.async.bulk.tensor.3d) as 76 x 12 boxes (x0-4 .., y0-2 ..) into a ring
-// of five shared-memory slots, one plane ahead of use, completion signalled on mbarriers.  Iteration `it` forms B^{n+1/2} on plane p = z0-1+it (tile, halo row y0-1, halo
-// column x0-1) and E^{n+1} on plane p-1, so one block barrier per plane suffices; B^{n+1/2}
-// lives in a small shared ring (B_x, B_y: 3 planes, B_z: 2 planes).  B^{n-1/2} is not staged:
-// each thread prefetches its own segment of the next plane from HBM into registers while the
-// current plane is computed.
+// of five shared-memory slots, one plane ahead of use, completion signalled on mbarriers.
+// Iteration `it` forms B^{n+1/2} on plane p = z0-1+it (tile, halo row y0-1, halo column x0-1) and
+// E^{n+1} on plane p-1, so one block barrier per plane suffices; B^{n+1/2} lives in a small shared
+// ring (B_x, B_y: 3 planes, B_z: 2 planes).  B^{n-1/2} is not staged: each thread prefetches its own
+// segment of the next plane from HBM into registers while the current plane is computed.
 //
 // Work per thread: W = 4 consecutive cells of one row, the same row in the B and the E phase.
 // A warp covers two whole rows.  Each stencil row a thread needs is read once as a 16-byte

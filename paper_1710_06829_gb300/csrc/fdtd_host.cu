@@ -1253,8 +1253,8 @@ static int pic_impl(fdtd_handle* h, int n, const fdtd_species* sp, int nsp) {
     h->hist_len = 0;   // a PIC cycle has no recorded adjoint
     // B^n once per cell (a pass of 36 B a cell in FP32) where the particles save more by it (24 of
     // 72 loads each); without the memory for it, once per particle.  Us a cycle, per particle / per
-    // cell, particles drifted by a cell: 128^3 and 0.5 per cell 183 / 177, 1 per cell 277 / 255, 2 per
-    // cell 461 / 401; 64^3 and 1 per cell 62 / 63, 2 per cell 83 / 80 (per cell now 4 to 6 % less).
+    // cell, both in blocks of 256, particles drifted by a cell: 128^3 and 0.5 per cell 183 / 177, 1 per
+    // cell 277 / 255, 2 per cell 461 / 401; 64^3 and 1 per cell 62 / 63, 2 per cell 83 / 80.
     const long long cells = (long long)g.nx * g.ny * g.nz;
     long long np = 0;
     for (int q = 0; q < nsp; ++q) np += sp[q].n;
@@ -1608,7 +1608,7 @@ int disp_omega_eval(const fdtd_coeffs* coeffs, double dt, const double dx[3], in
 // code running while a CUDA graph is being built on another stream of the same
 // device, a host that pre-reserves every byte of the GPU for its own pool, or a
 // plug-in that is not allowed to touch the allocator at all.  For them this entry
-// point runs the same three kernels as disp_norm_eval on a fixed scratch area
+// point runs the same two kernels as disp_norm_eval on a fixed scratch area
 // that the library declares statically on every device it is loaded on (512 KiB,
 // held until the process exits) instead of asking cudaMallocAsync for one.
 //
@@ -1622,7 +1622,7 @@ int disp_omega_eval(const fdtd_coeffs* coeffs, double dt, const double dx[3], in
 namespace {
 
 constexpr int kNoallocMaxN = 4096;              // per k-axis
-constexpr size_t kNoallocDoubles = 64 * 1024;   // 3*(3*4096) table + partials + results fit
+constexpr size_t kNoallocDoubles = 64 * 1024;   // tables (2 (3 x 4096) + 1028), partials, results fit
 constexpr int kNoallocMaxDevices = 64;
 
 static __device__ __align__(256) double g_norm_scratch[kNoallocDoubles];

@@ -6,14 +6,14 @@
 // marches z: the differences of E along each axis that its four cells share, and those that a later
 // plane needs again (kept in registers), are formed once, 14 a cell instead of 30; neighbouring
 // threads' differences are formed again rather than exchanged, so there is no barrier, and loads
-// come from L1.  About 77 FP64 instructions a cell and step, where the reference form takes 99.
+// come from L1.  77 FP64 instructions a cell and step (62 here, 15 in the Ampere kernel), where the
+// reference form takes 96.
 // Values and rounding order are those of dstar_diff / ampere_comp: bitwise the same fields.
 // Us a step, the kernels before (one tiled kernel with barriers where 64 x 8 tiles fit, else the
-// reference form) and these: 192 x 128 x 96 717 / 385, 100 x 90 x 80 199 / 124, 36^3 27 / 18,
-// 60 x 32 x 39 31 / 19,
-// 128^3 638 / 331 (0.157 ns a cell, 91 issue slots of the FP64 pipe).  A kernel that shares every
-// difference through shared memory (76 instructions, two barriers a plane) took 518 us at
-// 192 x 128 x 96: the pipe idles at the barriers.
+// reference form) and these: 192 x 128 x 96 717 / 386 (0.164 ns a cell), 100 x 90 x 80 199 / 125,
+// 36^3 27 / 18, 60 x 32 x 39 31 / 19, 128^3 638 / 355.  A kernel that shares every difference
+// through shared memory (76 instructions, two barriers a plane) took 518 us at 192 x 128 x 96: the pipe
+// idles at the barriers.
 #include <algorithm>
 
 #include "fdtd_seg64.cuh"

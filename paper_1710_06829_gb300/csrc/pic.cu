@@ -13,8 +13,9 @@
 //   J_x(i+1/2) - J_x(i-1/2) = -q W_x(i) / (dt dy dz),
 // so that (rho^{n+1} - rho^n)/dt + D.J^{n+1/2} = 0 holds to rounding (App. A numerical
 // continuity equation) and Gauss's law D.E = rho (Eq. divE) is kept.  A particle moves less
-// than a cell per step (|v| < c, c dt < dx on any stable grid), so per axis its old and new
-// supports fit the 4-node window floor(g0) - 1 .. floor(g0) + 2.
+// than a cell per step (|v| < c; dt^2 S <= 1 at k_a = pi / dx_a gives c dt <= dx_a where delta_a <= 0),
+// so per axis its old and new supports fit the 4-node window floor(g0) - 1 .. floor(g0) + 2.  A longer
+// move, which schemes with delta_a > 0 allow, is taken with the next cell's weights continued.
 //
 // Ampere's law is linear in J, so the cycle first forms E^{n+1} without the current (the
 // vacuum step kernel) and the push adds -dt J^{n+1/2} into its owned cells: no current
