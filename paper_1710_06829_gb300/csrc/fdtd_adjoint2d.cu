@@ -18,7 +18,7 @@
 // planes are one compensated FP32 sum a thread and axis); lambda is bitwise that of the 3D kernels.
 //
 // Bound: HBM for a large batch (60 B a cell), launch and latency for a small one.  Us a step, the 3D
-// kernel and this one: 512 x 512 x 32 148 / 97 (503 MB: 0.76 of the copy rate), 512 x 512 x 8 50 / 29,
+// kernel and this one: 512 x 512 x 32 148 / 97 (503 MB: 0.77 of the copy rate), 512 x 512 x 8 50 / 29,
 // 1024 x 1024 72 / 27, 192 x 40 x 70 38 / 23, 64 x 8 8.7 / 4.3.
 #include "fdtd_seg.cuh"
 

@@ -346,7 +346,7 @@ template void launch_bunch_table<double>(int, int, double, double, double, doubl
 // at a time, all loads before the stores, with one division by the row length a chunk.  The owner
 // of a chunk writes its images, so the dense array is read once.  256^3 FP32, six components, 805 MB
 // (119 us at the copy rate): unpacking took 556 us with one element and four 64-bit divisions a
-// thread, 147 us here; packing 416 us, now 159 us.
+// thread, 146 us here; packing 416 us, now 160 us.
 constexpr int COPY_THREADS = 256, COPY_ILP = 4;
 
 template <typename T>
