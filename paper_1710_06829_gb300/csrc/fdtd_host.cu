@@ -1445,11 +1445,15 @@ public:
     // The call's synchronisation: stream-ordered memory is given back before it, an area and its slot
     // after it and after the results are read.  Also where the call returns with the error e: kernels
     // that use the area may be queued all the same (an error that an earlier call of the thread left
-    // behind looks like a failed launch).
+    // behind looks like a failed launch).  In relaxed capture mode: while another thread captures a
+    // stream, the wait would otherwise be refused, with the kernels running, and end that capture.
     cudaError_t finish(cudaError_t e, double* out) {
         if (!ptr) return e;
         if (area_ < 0) cudaFreeAsync(ptr, st_);
+        cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+        cudaThreadExchangeStreamCaptureMode(&mode);
         const cudaError_t s = cudaStreamSynchronize(st_);
+        cudaThreadExchangeStreamCaptureMode(&mode);
         if (e == cudaSuccess) e = s;
         if (e == cudaSuccess && host_) memcpy(out, host_, 14 * sizeof(double));
         if (area_ >= 0) {

@@ -241,3 +241,26 @@ def test_temporal_blocking_on_ragged_grids(shape, slab, sponge):
         sm.close()
     for a, b in zip(*out):
         assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("name", ["disp_norm", "group_norm"])
+def test_norm_call_while_another_thread_captures(name):
+    """The call waits for its kernels, returns its value and leaves the capture as it was."""
+    import threading
+
+    from paper_1710_06829_gb300 import sim as S
+    args = (np.zeros((3, 3)), np.zeros(3), 0.4, [1.0, 1.0, 1.0], 3, (60, 50, 40))
+    ref = getattr(S, name)(*args)
+    st, side, got = torch.cuda.Stream(), torch.cuda.Stream(), []
+    x = torch.zeros(8, device="cuda")
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=st):
+        x.add_(1)
+        t = threading.Thread(target=lambda: got.append(getattr(S, name)(*args, stream=side)))
+        t.start()
+        t.join()
+        x.add_(1)
+    g.replay()
+    torch.cuda.synchronize()
+    assert got == [ref] and bool((x == 2).all())
